@@ -38,7 +38,7 @@ struct hadfl_handle {
   // fused round kernel scratch
   double *d_round_partials = nullptr;        // [round of a batch][2 N][blocks of the launch]
   double *d_round_group_partials = nullptr;  // [round of a batch][2 N][groups of kFinishGroup blocks]
-  unsigned int *d_round_ticket = nullptr;    // [round of a batch][1 + groups]: the round's ticket, one per group
+  unsigned int *d_round_ticket = nullptr;    // [1 + groups]: the launch's ticket, one per group of blocks
   float *d_round_stats = nullptr;            // [round of a batch][2 * kMaxDevices]
   int round_grid = 0;             // blocks of a launch with packs of 8 columns
   int round_grid_half_packs = 0;  // ... with packs of 4 columns (fp32 batches of one step per device)
@@ -480,9 +480,9 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
   const size_t round_vals = (size_t)kRoundBatchMax * 2 * (size_t)cfg->n_devices;
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_partials, sizeof(double) * round_vals * (size_t)scratch_grid));
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_group_partials, sizeof(double) * round_vals * n_groups));
-  HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_ticket, sizeof(unsigned int) * kRoundBatchMax * (1 + n_groups)));
+  HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_ticket, sizeof(unsigned int) * (1 + n_groups)));
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_stats, sizeof(float) * kRoundBatchMax * 2 * kMaxDevices));
-  HADFL_CUDA(h, cudaMemsetAsync(h->d_round_ticket, 0, sizeof(unsigned int) * kRoundBatchMax * (1 + n_groups),
+  HADFL_CUDA(h, cudaMemsetAsync(h->d_round_ticket, 0, sizeof(unsigned int) * (1 + n_groups),
                                 h->stream));
   HADFL_CUDA(h, cudaMemsetAsync(h->d_round_stats, 0, sizeof(float) * kRoundBatchMax * 2 * kMaxDevices, h->stream));
   HADFL_CUDA(h, cudaMemsetAsync(h->d_ticket, 0, sizeof(unsigned int), h->stream));

@@ -1,0 +1,47 @@
+"""The last-block finish of the statistics and of the fused round at the sizes where its loops change
+shape: block counts around the group size (128 blocks), around a warp's stride over the partial sums
+(32 lanes x 4 loads), one block, and more than one group; a launch with one round and one with several.
+The sums must match a double-precision sum over the arena as it stands afterwards.  Bound: a value is
+added to at most 8 others in a thread, then once across lanes and over 8 warps in fp32, all terms
+positive: relative error <= (8 + 1 + 8) * 2^-24 = 1.0e-6, and the output's own rounding 2^-24."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_common import require_gpu
+from paper_2111_08274_b200 import runtime, workloads
+from paper_2111_08274_b200.workloads import Workload
+
+pytestmark = pytest.mark.gpu
+BOUND = 18 * 2.0 ** -24
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def sums(arena, ref):
+    w = arena.w[:, : arena.wl.n_params].double()
+    return (w * w).sum(1).cpu().numpy(), ((w - w[ref]) ** 2).sum(1).cpu().numpy()
+
+
+def check(got, want):
+    assert np.allclose(got[0], want[0], rtol=BOUND, atol=0)
+    # distances are sums over fp32 differences, each rounded once more before it is squared
+    assert np.allclose(got[1], want[1], rtol=BOUND + 2.0 ** -23, atol=0)
+
+
+@pytest.mark.parametrize("blocks", [1, 2, 31, 32, 33, 127, 128, 129, 255, 257, 300])
+@pytest.mark.parametrize("n,k,extra", [(2, 1, 0), (3, 2, 1), (17, 16, -1)])
+def test_sums_over_block_counts(blocks, n, k, extra):
+    wl = Workload("fin", n, 2048 * blocks + extra, k, 1, "fixed", (1,) * n, grad_std=1e-2,
+                  seed=workloads.BASE_SEED + blocks)
+    arena = runtime.Arena(wl)
+    sel = arena.run_round_fused(0)                       # a launch of one round
+    check(arena.h.stats_read(), sums(arena, int(sel[0])))
+    sel = arena.run_rounds_fused(1, 3)[-1]               # a launch of three
+    check(arena.h.stats_read(), sums(arena, int(sel[0])))
+    ref = n - 1
+    check(arena.h.stats(ref), sums(arena, ref))          # the statistics kernel
+    arena.close()
