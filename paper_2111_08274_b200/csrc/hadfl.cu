@@ -89,6 +89,7 @@ constexpr size_t kBatchSmallArenaBytes = (size_t)64 << 20;  // arenas up to this
 constexpr int kRowPerBlockMaxSteps = 2;  // up to this many steps per device a launch is memory-bound: the local update
                                          // then takes one row per block (fp32), the fused round prefetches rows (bf16)
 constexpr int kStatsU = 4;  // 16-byte packs per thread and chunk in the statistics kernel
+constexpr int64_t kRowsGridCap = 4096;         // most blocks of a fused-round launch with a warp per row
 constexpr int64_t kRoundGridCap = 16384;  // most blocks of a fused-round launch (bounds its scratch: 8 MB)
 
 // Columns per thread in the local-update and fused-round kernels: two Philox blocks (two 16-byte
@@ -256,8 +257,67 @@ int launch_local_step(hadfl_handle *h, const LocalStepArgs &a, float lr) {
   });
 }
 
+// Whether a launch of n_rounds fused rounds takes the form with a warp per row (k_round_rows): where the
+// row walk of k_round leaves most of the chip idle.  k_round has one block per 2048 columns and takes a
+// time that grows with the number of rows until those blocks fill the chip; the rows form's grows with
+// all the work.  Measured, us per round, row walk / rows form (steps 1, then 8 per device):
+//   8 rounds per launch: 8 devices 131,072 parameters 8.3 / 5.1, 25.6 / 12.3; 524,288: 12.4 / 10.6, 39.4 /
+//     33.3; 16 devices 65,536: 14.4 / 5.4, 49.4 / 12.8; 262,144: 14.7 / 11.5, 49.5 / 35.6; 524,288 with steps
+//     1,1,2,2,4,4,8,8: 43 / 48; 32 devices 131,072: 26.6 / 14.3, 96.9 / 45.3; 200,000 (16 selected) with
+//     steps 1..4: 47.7 / 47.9
+//   one round per launch: 8 devices 131,072: 12.7 / 12.0, 28.8 / 17.8; 200,000: 12.7 / 14.7, 29.1 / 22.9;
+//     16 devices 65,536: 18.0 / 12.4, 51.3 / 18.8; 131,072: 18.6 / 17.9, 51.6 / 28.8; 262,144: 18.8 / 26.8;
+//     32 devices 131,072 (16 selected): 31.1 / 37.2
+bool rows_form(const hadfl_handle *h, int n_rounds) {
+  const int64_t P = h->cfg.n_params, work = h->cfg.n_devices * P;
+  return n_rounds > 1 ? work <= ((int64_t)1 << 22) : P <= ((int64_t)1 << 17) && work <= ((int64_t)1 << 21);
+}
+
+// Rows form: tiles of a block (at least 8 warps) and blocks of a launch.
+int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
+int64_t rows_grid(int n_devices, int64_t n_params) {
+  constexpr int kCols = 32 * StepPack<float>::E;
+  const int64_t tiles = (n_params + kCols - 1) / kCols;
+  const int64_t blocks = (tiles + rows_groups(n_devices) - 1) / rows_groups(n_devices);
+  return blocks < kRowsGridCap ? blocks : kRowsGridCap;
+}
+
+template <int NR>
+int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
+  return for_storage(h, [&](auto wt, auto mt, auto rm) {
+    using WT = typename decltype(wt)::type;
+    using MT = typename decltype(mt)::type;
+    constexpr int E = StepPack<WT>::E;
+    RowsBatch<NR> q;
+    q.n = h->cfg.n_devices;
+    q.k = b.round[0].k;
+    q.n_rounds = b.n_rounds;
+    q.groups = rows_groups(q.n);
+    q.beta = b.round[0].beta;
+    q.one_minus_beta = b.round[0].one_minus_beta;
+    for (int r = 0; r < b.n_rounds; ++r) {
+      const RoundArgs &a = b.round[r];
+      q.write_all[r] = a.write_all;
+      memcpy(q.a[r], a.a, sizeof(a.a));
+      for (int j = 0; j < q.n; ++j) q.s[r][a.r[j].row] = RowsStep{a.r[j].steps, a.r[j].base_lo, a.r[j].r1_c2, j};
+    }
+    const int grid = (int)rows_grid(q.n, h->cfg.n_params);
+    const size_t smem = rows_shared_bytes<WT, E>(q.groups, q.n, q.k, b.n_rounds);
+    const RoundScratch scratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket,
+                               h->d_round_stats, h->d_stats};
+    auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR>;
+    if (smem > 48 * 1024)  // more than 16 selected devices
+      HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<grid, q.groups * q.n * 32, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->stride, h->cfg.n_params, h->keys,
+                                                           step_consts(h, lr), scratch, q);
+    h->last_launch_pack = E;
+    return check_launch(h);
+  });
+}
+
 template <int NR>
 int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
+  if (rows_form(h, b.n_rounds)) return launch_round_rows<NR>(h, b, lr);
   return for_storage(h, [&](auto wt, auto mt, auto rm) {
     using WT = typename decltype(wt)::type;
     using MT = typename decltype(mt)::type;
@@ -475,7 +535,9 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
     h->round_half_packs = cfg->dtype == HADFL_DTYPE_FP32 && resident_rows <= 0.8 * l2_bytes &&
                           (size_t)cfg->n_devices * (size_t)cfg->n_params * 8 > kBatchSmallArenaBytes;
   }
-  const int scratch_grid = h->round_grid_half_packs > h->round_grid ? h->round_grid_half_packs : h->round_grid;
+  int scratch_grid = h->round_grid_half_packs > h->round_grid ? h->round_grid_half_packs : h->round_grid;
+  if (rows_grid(cfg->n_devices, cfg->n_params) > scratch_grid)
+    scratch_grid = (int)rows_grid(cfg->n_devices, cfg->n_params);
   const size_t n_groups = (size_t)((scratch_grid + kFinishGroup - 1) / kFinishGroup);
   const size_t round_vals = (size_t)kRoundBatchMax * 2 * (size_t)cfg->n_devices;
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_partials, sizeof(double) * round_vals * (size_t)scratch_grid));

@@ -132,6 +132,17 @@ __device__ __forceinline__ void unpack(const RawPack<__nv_bfloat16, 4> &r, float
   bf16x2_to_floats(r.q.y, v[2], v[3]);
 }
 
+// fp32 values as a pack in storage form (bf16: to nearest even).
+template <int E>
+__device__ __forceinline__ void pack_raw(const float (&v)[E], RawPack<float, E> &r) {
+#pragma unroll
+  for (int i = 0; i < E; ++i) r.v[i] = v[i];
+}
+__device__ __forceinline__ void pack_raw(const float (&v)[8], RawPack<__nv_bfloat16, 8> &r) {
+  r.q = make_uint4(floats_to_bf16x2(v[0], v[1]), floats_to_bf16x2(v[2], v[3]), floats_to_bf16x2(v[4], v[5]),
+                   floats_to_bf16x2(v[6], v[7]));
+}
+
 // `at` points to the first element of the pack.  live == E: vector load; otherwise (the ragged
 // last pack of a row) element by element, dead lanes read as 0.
 template <int E>
@@ -1199,6 +1210,209 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
     } else if (j >= a.k) {
       put(which * n_dev + a.r[j].row, (float)sum);
     }
+  });
+}
+
+// ------------------------------------------------------------------------------------------
+// Fused rounds of small vectors: a warp per row.  The rows of a tile of 32 * E columns are spread over
+// the warps of a group instead of being walked by one thread, and stay in registers through all rounds
+// of a batch.  Per round a warp runs its row's steps; the selected warps leave their rows in shared
+// memory; one barrier of the group; every warp then forms the aggregate for itself (in draw order, as
+// k_round does) and takes its statistics against it.  Two buffers in turn make one barrier per round
+// enough: a warp that writes round r + 2 has passed the barrier of round r + 1, which no warp reaches
+// before it has read round r.  Parameters and momentum come out bit-identical to k_round.
+// What bounds a round here is latency: that of the slowest row (k_round: of all rows one after the
+// other) plus the hand-over, and there are n times as many warps to fill the chip.
+// On large vectors the waits at the barrier, where all warps of a group are in the same phase, cost more
+// than registers save; there k_round is the faster one (the host decides: see rows_form).
+// A row moves to another warp from block to block, so that the heavy rows meet all SM sub-partitions.
+// Sums of a row: fp32 within the tile (pack in order, then a fixed tree), fp64 beyond.
+// ------------------------------------------------------------------------------------------
+constexpr int kRowsMaxThreads = 1024;
+
+struct RowsStep {  // one device in one round
+  int32_t steps;
+  uint32_t base_lo, r1_c2;  // as in RowStep
+  int32_t visit;            // position in the draw (0 .. k - 1: selected), or k and above
+};
+template <int NR>
+struct RowsBatch {
+  int32_t n, k, n_rounds;
+  int32_t groups;             // tiles that a block has in hand at a time
+  float beta, one_minus_beta;
+  int32_t write_all[NR];      // as in RoundArgs
+  float a[NR][kMaxDevices];   // aggregation weights in draw order
+  __align__(16) RowsStep s[NR][kMaxDevices];
+};
+
+// A selected row of a tile in shared memory: [plane of 16 (or 8) bytes][lane].
+template <typename WT, int E>
+struct SelectedRow {
+  static constexpr int kPackBytes = E * (int)sizeof(WT);
+  using Unit = typename std::conditional<kPackBytes >= 16, uint4, uint2>::type;
+  static constexpr int kPlanes = kPackBytes / (int)sizeof(Unit);
+  static constexpr int kBytes = kPackBytes * 32;
+  static __device__ __forceinline__ void load(const char *row, int lane, RawPack<WT, E> &r) {
+    Unit u[kPlanes];
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i) u[i] = reinterpret_cast<const Unit *>(row)[i * 32 + lane];
+    memcpy(&r, u, kPackBytes);
+  }
+  static __device__ __forceinline__ void store(char *row, int lane, const RawPack<WT, E> &r) {
+    Unit u[kPlanes];
+    memcpy(u, &r, kPackBytes);
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i) reinterpret_cast<Unit *>(row)[i * 32 + lane] = u[i];
+  }
+};
+
+// Dynamic shared memory of a block: [group][2][k] selected rows, [group][round][n][2] row sums.
+template <typename WT, int E>
+constexpr size_t rows_selected_bytes(int k) { return (size_t)2 * k * SelectedRow<WT, E>::kBytes; }
+template <typename WT, int E>
+constexpr size_t rows_shared_bytes(int groups, int n, int k, int rounds) {
+  return groups * (rows_selected_bytes<WT, E>(k) + sizeof(double) * 2 * n * rounds);
+}
+
+template <typename WT, typename MT, typename Gen, int E, int RM, int NR>
+__global__ void __launch_bounds__(kRowsMaxThreads)
+k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_params,
+             PhiloxKeys keys, StepConsts k, RoundScratch scratch, const __grid_constant__ RowsBatch<NR> b) {
+  using Sel = SelectedRow<WT, E>;
+  extern __shared__ __align__(16) char s_rows[];
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = b.n, n_sel = b.k, groups = b.groups;
+  const int n_rounds = NR == 1 ? 1 : b.n_rounds;
+  const int n_vals = n_rounds * 2 * n;
+  const int group = warp / n;
+  const int row = (warp - group * n + (int)blockIdx.x) % n;
+  char *sel = s_rows + group * 2 * n_sel * Sel::kBytes;
+  double *all_sums = reinterpret_cast<double *>(s_rows + groups * 2 * n_sel * Sel::kBytes);
+  double *sums = all_sums + group * n_vals + 2 * row;  // each owned by the warp of that row
+  for (int t = threadIdx.x; t < groups * n_vals; t += blockDim.x) all_sums[t] = 0.0;
+  RowStep rs;
+  rs.row = row;
+  {
+    const uint64_t dp = (uint64_t)kPhiloxM1 * (uint32_t)row;
+    rs.r1_c0 = (uint32_t)(dp >> 32) ^ keys.a[0];
+    rs.r1_c1 = (uint32_t)dp;
+  }
+  __syncthreads();
+
+  const int64_t n_packs = (n_params + E - 1) / E;
+  const int64_t n_tiles = (n_packs + 31) / 32;
+  for (int64_t tile = (int64_t)blockIdx.x * groups + group; tile < n_tiles; tile += (int64_t)gridDim.x * groups) {
+    auto do_tile = [&](auto all_full) {
+      const int64_t p = tile * 32 + lane;
+      const int live = decltype(all_full)::value ? E : live_of(n_params, p, E);
+      const GroupProducts<E / 4> gp(p);
+      WT *wp = w + row * stride + p * E;
+      MT *mp = m + row * stride + p * E;
+      float wv[E], mv[E];
+      {
+        RawPack<WT, E> rw;
+        RawPack<MT, E> rm;
+        ld_raw(wp, live, rw);
+        ld_raw(mp, live, rm);
+        unpack(rw, wv);
+        unpack(rm, mv);
+      }
+      bool w_changed = false, m_changed = false;
+#pragma unroll 1
+      for (int r = 0; r < n_rounds; ++r) {
+        const RowsStep &st = b.s[r][row];
+        rs.steps = st.steps;
+        rs.base_lo = st.base_lo;
+        rs.r1_c2 = st.r1_c2;
+        const int j = st.visit, write_all = b.write_all[r];
+        if (rs.steps > 0) {
+          sgd_steps<Gen, E / 4>(wv, mv, gp, rs, keys, k);
+          if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, rs, keys);
+#pragma unroll
+          for (int i = 0; i < E; ++i) {
+            wv[i] = as_stored(wv[i], w);
+            mv[i] = as_stored(mv[i], m);
+          }
+          if (live < E) {  // lanes beyond the end of the vector stay 0 in the sums
+#pragma unroll
+            for (int i = 0; i < E; ++i) wv[i] = i < live ? wv[i] : 0.f;
+          }
+          w_changed = m_changed = true;
+        }
+        char *buf = sel + (r & 1) * n_sel * Sel::kBytes;
+        if (j < n_sel) {
+          RawPack<WT, E> rw;
+          pack_raw(wv, rw);
+          Sel::store(buf + j * Sel::kBytes, lane, rw);
+        }
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(n * 32) : "memory");
+        float acc[E];
+        {
+          RawPack<WT, E> rw;
+          float v[E];
+          Sel::load(buf, lane, rw);
+          unpack(rw, v);
+          const float a0 = b.a[r][0];
+#pragma unroll
+          for (int i = 0; i < E; ++i) acc[i] = __fmul_rn(a0, v[i]);
+          for (int t = 1; t < n_sel; ++t) {
+            Sel::load(buf + t * Sel::kBytes, lane, rw);
+            unpack(rw, v);
+            const float a_t = b.a[r][t];
+#pragma unroll
+            for (int i = 0; i < E; ++i) acc[i] = fmaf(a_t, v[i], acc[i]);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < E; ++i) acc[i] = as_stored(acc[i], w);
+        if (j < n_sel || write_all == 1) {
+#pragma unroll
+          for (int i = 0; i < E; ++i) wv[i] = acc[i];
+          w_changed = true;
+        } else if (write_all == 2) {
+#pragma unroll
+          for (int i = 0; i < E; ++i)
+            wv[i] = as_stored(fmaf(b.beta, acc[i], __fmul_rn(b.one_minus_beta, wv[i])), w);
+          w_changed = true;
+        }
+        float n2 = 0.f, d2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          const float d = wv[i] - acc[i];
+          n2 = fmaf(wv[i], wv[i], n2);
+          d2 = fmaf(d, d, d2);
+        }
+        const bool upper = (lane & 16) != 0;
+        float v = (upper ? d2 : n2) + __shfl_xor_sync(0xFFFFFFFFu, upper ? n2 : d2, 16);
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        if ((lane & 15) == 0) sums[r * 2 * n + (lane >> 4)] += (double)v;  // lower half-warp norms, upper distances
+      }
+      if (w_changed) st_pack_any(wp, 0, live, wv);
+      if (m_changed) st_pack_any(mp, 0, live, mv);
+      // the next tile's first round must not overwrite a buffer that is still being read
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(n * 32) : "memory");
+    };
+    if ((tile + 1) * 32 * E <= n_params)
+      do_tile(std::true_type{});
+    else
+      do_tile(std::false_type{});
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < n_vals; t += blockDim.x) {
+    double d = 0.0;
+    for (int g = 0; g < groups; ++g) d += all_sums[g * n_vals + t];
+    double *at = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
+    if (access_ok(at, 8)) *at = d;
+  }
+  // one two-level finish over all rounds of the batch (one fence and one ticket per block)
+  finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
+                   [&](int t, double sum) {
+    const int r = t / (2 * n), v = t - r * 2 * n, at = (v & 1) * n + (v >> 1);  // [norms of the rows][distances]
+    float *out_r = scratch.out_rounds + r * 2 * kMaxDevices;
+    if (access_ok(out_r + at, 4)) out_r[at] = (float)sum;
+    if (r + 1 == n_rounds && access_ok(scratch.out + at, 4)) scratch.out[at] = (float)sum;
   });
 }
 
