@@ -25,6 +25,9 @@ struct hadfl_handle {
   cudaStream_t stream = nullptr;
   int device = 0;
   int sm_count = 0;
+  int l2_bytes = 0;
+  size_t smem_per_sm = 0;
+  size_t resident_arena_bytes = 0;  // batches on arenas beyond this are resident on the SMs
   PhiloxKeys keys;
   uint32_t version[kMaxDevices];
   uint64_t step_count[kMaxDevices];
@@ -63,6 +66,9 @@ namespace {
 
 inline size_t elem_size(const hadfl_handle *h) { return h->cfg.dtype == HADFL_DTYPE_BF16 ? 2 : 4; }
 inline size_t m_elem_size(const hadfl_handle *h) { return h->cfg.m_dtype == HADFL_DTYPE_BF16 ? 2 : 4; }
+inline size_t arena_bytes(const hadfl_handle *h) {
+  return (size_t)h->cfg.n_devices * (size_t)h->cfg.n_params * (elem_size(h) + m_elem_size(h));
+}
 
 // Calls f(parameter storage type, momentum storage type, rounding mode) for the handle's storage
 // configuration: fp32 / fp32, or bf16 parameters with fp32 or bf16 momentum, each rounded to
@@ -88,6 +94,7 @@ int for_storage(const hadfl_handle *h, F &&f) {
 constexpr size_t kBatchSmallArenaBytes = (size_t)64 << 20;  // arenas up to this size are bound by launches, not bytes
 constexpr int kRowPerBlockMaxSteps = 2;  // up to this many steps per device a launch is memory-bound: the local update
                                          // then takes one row per block (fp32), the fused round prefetches rows (bf16)
+constexpr size_t kSmemReserve = 1024 + 64;  // per block: what the system takes, and the kernel's own variables
 constexpr int kStatsU = 4;  // 16-byte packs per thread and chunk in the statistics kernel
 constexpr int64_t kRowsGridCap = 4096;         // most blocks of a fused-round launch with a warp per row
 constexpr int64_t kRoundGridCap = 16384;  // most blocks of a fused-round launch (bounds its scratch: 8 MB)
@@ -315,9 +322,107 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
   });
 }
 
+// Whether a batch takes the resident form (k_rounds_resident) instead of the row walk through L2: on arenas
+// well beyond the L2, where the row walk pays HBM and L2 for every round, and on small ones with few
+// devices.  Measured, us per round, row walk / resident (one step, then 1..4 steps per device): 8 devices
+// 1,048,576 parameters 22.3 / 16.3, 29.0 / 26.3; 2.5 M 36.8 / 32.8, 70.8 / 56.4; 16 devices 524,288: 21.9 /
+// 23.4, 32.6 / 35.2; 1,048,576 (the arena is about the L2): 34.7 / 37 and more; 32 devices 262,144: 26.9 / 37.
+// Large arenas of up to 16 devices gain with any number of rounds (1.5e8 parameters in all: 2 rounds 0.98 .. 1.12
+// times the speed, 8 rounds 1.02 .. 1.37).  With more devices half the rows and more stay in L2 while few
+// blocks share an SM, so the form has to save several rounds' traffic: 32 devices, one step, 2 / 3 / 4 /
+// 8 rounds 435 / 436 / 435 / 440 -> 487 / 422 / 383 / 352; two steps 411 .. 415 -> 561 / 511 / 485 / 460; 24
+// devices, two steps, 2 / 4 / 6 / 8 rounds 414 .. 416 -> 472 / 420 / 398 / 396.
+bool resident_form(const hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b) {
+  const size_t arena = arena_bytes(h);
+  const int n = h->cfg.n_devices;
+  if (arena <= kBatchSmallArenaBytes) return n <= 8;
+  if (arena <= h->resident_arena_bytes) return false;
+  if (n <= 16) return true;
+  int64_t sum_steps = 0;
+  for (int r = 0; r < b.n_rounds; ++r)
+    for (int j = 0; j < n; ++j) sum_steps += b.round[r].r[j].steps;
+  return 2 * sum_steps <= 3 * (int64_t)n * b.n_rounds ? b.n_rounds >= 4 : n <= 24 && b.n_rounds >= 6;
+}
+
+int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b, float lr) {
+  return for_storage(h, [&](auto wt, auto mt, auto rm) {
+    using WT = typename decltype(wt)::type;
+    using MT = typename decltype(mt)::type;
+    constexpr int kWords = 2 * (int)sizeof(MT);
+    ResidentBatch q;
+    const int n = q.n = h->cfg.n_devices;
+    q.k = b.round[0].k;
+    q.n_rounds = b.n_rounds;
+    q.beta = b.round[0].beta;
+    q.one_minus_beta = b.round[0].one_minus_beta;
+    int64_t sum_steps = 0;
+    for (int r = 0; r < b.n_rounds; ++r) {
+      const RoundArgs &a = b.round[r];
+      q.write_all[r] = a.write_all;
+      memcpy(q.a[r], a.a, sizeof(a.a));
+      int n_stepping = 0;
+      for (int j = 0; j < n; ++j) {
+        const RowStep &rs = a.r[j];
+        q.draw[r][j] = rs.row;
+        q.w_off[rs.row] = rs.w_off;
+        q.m_off[rs.row] = rs.m_off;
+        q.s[r][rs.row] = RowsStep{rs.steps, rs.base_lo, rs.r1_c2, j};
+        q.r1_c0[rs.row] = rs.r1_c0;
+        q.r1_c1[rs.row] = rs.r1_c1;
+        if (rs.steps == 0) continue;
+        sum_steps += rs.steps;
+        int at = n_stepping++;
+        for (; at > 0 && q.s[r][q.order[r][at - 1]].steps < rs.steps; --at) q.order[r][at] = q.order[r][at - 1];
+        q.order[r][at] = rs.row;
+      }
+      q.n_stepping[r] = n_stepping;
+    }
+    const int64_t mean_steps_x2 = 2 * sum_steps / ((int64_t)n * b.n_rounds);
+    // Blocks per SM.  With more than two steps per device on average the launch is bound by arithmetic, and 6
+    // blocks are the fastest whatever they leave to the L2.  Otherwise the most, up to 5 (6, where those find
+    // room for as many rows), whose rows in the arena stay within 55 % of the L2: 72 MB of them, with 16
+    // devices and 6 blocks, already came back from HBM (478 against 431 us per round).
+    const size_t sums = resident_sums_bytes(n, b.n_rounds);
+    constexpr size_t kRowBytes = RowStore<WT>::kRowBytes;
+    auto rows_on_chip = [&](int blocks) {
+      int columns = 512;
+      while (columns * blocks > 512) columns /= 2;
+      const int room = (int)((h->smem_per_sm / blocks - kSmemReserve - sums) / kRowBytes);
+      const int fit = columns / kWords < room ? columns / kWords : room;
+      return fit < n ? fit : n;
+    };
+    auto in_l2 = [&](int blocks) {
+      return (double)(n - rows_on_chip(blocks)) * blocks * h->sm_count * kResidentThreads * 8.0 * (sizeof(WT) + sizeof(MT));
+    };
+    int blocks_per_sm = kResidentMaxBlocks;
+    if (mean_steps_x2 <= 4) {
+      if (rows_on_chip(blocks_per_sm) < rows_on_chip(blocks_per_sm - 1)) --blocks_per_sm;
+      while (blocks_per_sm > 2 && in_l2(blocks_per_sm) > 0.55 * h->l2_bytes) --blocks_per_sm;
+    }
+    q.n_on_chip = rows_on_chip(blocks_per_sm);
+    // As much shared memory as keeps the number of blocks at that.
+    size_t smem = q.n_on_chip * kRowBytes + sums;
+    const size_t floor_bytes = h->smem_per_sm / (blocks_per_sm + 1) - kSmemReserve + 1024;
+    if (smem < floor_bytes && blocks_per_sm < kResidentMaxBlocks) smem = floor_bytes;
+    const int64_t chunks = (h->cfg.n_params + 8 * kResidentThreads - 1) / (8 * kResidentThreads);
+    const int grid = (int)(chunks < kRoundGridCap ? chunks : kRoundGridCap);
+    const RoundScratch scratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket,
+                               h->d_round_stats, h->d_stats};
+    auto kernel = q.n_on_chip == n ? k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, true>
+                                   : k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, false>;
+    HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<grid, kResidentThreads, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->cfg.n_params, h->keys,
+                                                        step_consts(h, lr), scratch, q);
+    h->last_launch_pack = 8;
+    return check_launch(h);
+  });
+}
+
 template <int NR>
 int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
   if (rows_form(h, b.n_rounds)) return launch_round_rows<NR>(h, b, lr);
+  if constexpr (NR > 1)
+    if (resident_form(h, b)) return launch_rounds_resident(h, b, lr);
   return for_storage(h, [&](auto wt, auto mt, auto rm) {
     using WT = typename decltype(wt)::type;
     using MT = typename decltype(mt)::type;
@@ -529,10 +634,13 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
     // device, 8 rounds per launch: 151 against 181 us per round with 8 devices at the ResNet-18 size,
     // 447 against 600 us with 16 devices and 2^24 parameters; with 32 devices - 155 MB of rows -
     // 2065 against 1943 us, and 19.1 against 17.5 us at 2^18 parameters, where launches are the cost).
-    int l2_bytes = 0;
-    HADFL_CUDA(h, cudaDeviceGetAttribute(&l2_bytes, cudaDevAttrL2CacheSize, h->device));
+    HADFL_CUDA(h, cudaDeviceGetAttribute(&h->l2_bytes, cudaDevAttrL2CacheSize, h->device));
+    int smem_per_sm = 0;
+    HADFL_CUDA(h, cudaDeviceGetAttribute(&smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
+    h->smem_per_sm = (size_t)smem_per_sm;
+    h->resident_arena_bytes = (size_t)h->l2_bytes / 8 * 9;
     const double resident_rows = 4.0 * h->sm_count * cfg->n_devices * (kThreads * 4.0) * 8.0;
-    h->round_half_packs = cfg->dtype == HADFL_DTYPE_FP32 && resident_rows <= 0.8 * l2_bytes &&
+    h->round_half_packs = cfg->dtype == HADFL_DTYPE_FP32 && resident_rows <= 0.8 * h->l2_bytes &&
                           (size_t)cfg->n_devices * (size_t)cfg->n_params * 8 > kBatchSmallArenaBytes;
   }
   int scratch_grid = h->round_grid_half_packs > h->round_grid ? h->round_grid_half_packs : h->round_grid;
@@ -855,16 +963,19 @@ int round_by_separate_calls(hadfl_handle *h, const int32_t *device_ids, const in
   return rc;
 }
 
-// Whether hadfl_rounds may put a planned round into a launch together with its neighbours.  A
-// batch pays where a round is bound by memory or by the launch itself: every device runs at most
-// kRowPerBlockMaxSteps steps, or the arena is small against the L2.  With more steps per device
-// the rounds are bound by arithmetic and the batch's indexed arguments cost what L2 saves
-// (measured: 0 ... -3 %), so those rounds are launched one by one; the same holds for stochastic
-// rounding, which draws a second random block per pack and call (measured: -3 ... -5 %).
+// Whether hadfl_rounds may put a planned round into a launch together with its neighbours.
+//   - Arenas of at most 64 MiB, where launches and latency are the cost: always.
+//   - Where batches are resident and at most 16 devices leave most rows on the SM: always (16 devices, 14.7 M,
+//     steps 1,1,2,2,4,4,8,8: 863 -> 822 us per round, bf16 parameters 859 -> 816; 8 devices, 11.2 M, 1..8 steps
+//     360 -> 345; but 32 devices, 12 M, 1..4 steps 1165 -> 1269).
+//   - Else rounds of at most two steps per device, which are bound by memory, and only with rounding to nearest
+//     even: stochastic rounding draws a second random block per pack and call (row walk -3 ... -5 %; resident
+//     with 24 and 32 devices -6 ... +2 %).  With more steps the row walk gains nothing (0 ... -3 %).
 bool batchable(const hadfl_handle *h, const RoundPlan &pl) {
   if (h->round_batch <= 1) return false;
-  const size_t arena = (size_t)h->cfg.n_devices * (size_t)h->cfg.n_params * (elem_size(h) + m_elem_size(h));
+  const size_t arena = arena_bytes(h);
   if (arena <= kBatchSmallArenaBytes) return true;
+  if (arena > h->resident_arena_bytes && h->cfg.n_devices <= 16) return true;
   if (h->cfg.rounding == HADFL_ROUND_STOCHASTIC) return false;
   for (int i = 0; i < h->cfg.n_devices; ++i)
     if (pl.row_steps[i] > kRowPerBlockMaxSteps) return false;

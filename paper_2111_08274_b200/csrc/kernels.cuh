@@ -192,6 +192,31 @@ __device__ __forceinline__ void ld_raw(const __nv_bfloat16 *at, int live, RawPac
     r.q.y = ld_bf16_bits(at, 2, live) | (ld_bf16_bits(at, 3, live) << 16);
   }
 }
+// The same pack back to memory as it is.
+template <int E>
+__device__ __forceinline__ void st_raw(float *at, int live, const RawPack<float, E> &r) {
+  if (!access_ok(at, 4 * (size_t)live)) return;
+  if (live == E) {
+#pragma unroll
+    for (int i = 0; i < E / 4; ++i)
+      *reinterpret_cast<float4 *>(at + 4 * i) = make_float4(r.v[4 * i], r.v[4 * i + 1], r.v[4 * i + 2], r.v[4 * i + 3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < E; ++i)
+      if (i < live) at[i] = r.v[i];
+  }
+}
+__device__ __forceinline__ void st_raw(__nv_bfloat16 *at, int live, const RawPack<__nv_bfloat16, 8> &r) {
+  if (!access_ok(at, 2 * (size_t)live)) return;
+  if (live == 8) {
+    *reinterpret_cast<uint4 *>(at) = r.q;
+  } else {
+    const uint32_t words[4] = {r.q.x, r.q.y, r.q.z, r.q.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < live) reinterpret_cast<unsigned short *>(at)[i] = (unsigned short)(words[i / 2] >> (16 * (i & 1)));
+  }
+}
 template <typename WT, int E>
 __device__ __forceinline__ void zero_raw(RawPack<WT, E> &r) {
   memset(&r, 0, sizeof(r));
@@ -437,6 +462,58 @@ __device__ __forceinline__ void sgd_update_pair(float &w0, float &w1, float &m0,
 // The launch is bound by the issue slot with several steps per device, and this takes 22 of 155
 // warp instructions out of a step of an 8-parameter pack (measured: K1 -3 ... -4 %, fused round
 // -4 ... -5 %).
+// The gradient noise of step e for the NB column groups of a pack: nz[b] = grad_std * (z0, z1), (z2, z3).
+template <typename Gen, int NB>
+__device__ __forceinline__ void step_noise(float2 (&nz)[NB][2], int e, const uint32_t (&c2_first)[NB],
+                                           const GroupProducts<NB> &gp, const RowStep &rs, const PhiloxKeys &keys,
+                                           const StepConsts &k) {
+  const uint32_t c0_first = rs.r1_c0 ^ (rs.base_lo + (uint32_t)e);
+  uint32_t x[NB][4];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    x[b][0] = c0_first; x[b][1] = rs.r1_c1; x[b][2] = c2_first[b]; x[b][3] = gp.lo[b];
+  }
+#pragma unroll
+  for (int r = 1; r < 10; ++r)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) philox_round(x[b][0], x[b][1], x[b][2], x[b][3], keys.a[r], keys.b[r]);
+  float2 r2[NB];  // squared radii of the block's two pairs
+  uint32_t top = 0;
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    r2[b] = Gen::radius2_pair(x[b][0], x[b][2], k.lg_scale);
+    top = max(top, max(x[b][0], x[b][2]));
+  }
+  if (Gen::needs_series(top)) {  // about once in 250 steps of a pack
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      if (Gen::needs_series(x[b][0])) r2[b].x = r2_next_to_one(x[b][0], k.scale2);
+      if (Gen::needs_series(x[b][2])) r2[b].y = r2_next_to_one(x[b][2], k.scale2);
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const float2 theta = Gen::angle_pair(x[b][1], x[b][3]);
+    nz[b][0] = Gen::finish_pair(r2[b].x, theta.x);
+    nz[b][1] = Gen::finish_pair(r2[b].y, theta.y);
+  }
+}
+
+template <int NB>
+__device__ __forceinline__ void step_update(float (&w)[4 * NB], float (&m)[4 * NB], const float2 (&nz)[NB][2],
+                                            const StepConsts &k) {
+  const float2 wd2 = make_float2(k.wd, k.wd), mu2 = make_float2(k.mu, k.mu);
+  const float2 neg_lr2 = make_float2(k.neg_lr, k.neg_lr);
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    sgd_update_pair(w[4 * b], w[4 * b + 1], m[4 * b], m[4 * b + 1], nz[b][0], wd2, mu2, neg_lr2);
+    sgd_update_pair(w[4 * b + 2], w[4 * b + 3], m[4 * b + 2], m[4 * b + 3], nz[b][1], wd2, mu2, neg_lr2);
+  }
+}
+
+// All steps of a row.  The loop is not unrolled: the copies
+// would compute the step-independent products of the generator more than once (fused round 584 -> 578
+// us at 8 steps per device, ResNet-18 size).
 template <typename Gen, int NB>
 __device__ __forceinline__ void sgd_steps(float (&w)[4 * NB], float (&m)[4 * NB],
                                           const GroupProducts<NB> &gp, const RowStep &rs,
@@ -444,41 +521,11 @@ __device__ __forceinline__ void sgd_steps(float (&w)[4 * NB], float (&m)[4 * NB]
   uint32_t c2_first[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) c2_first[b] = gp.hi[b] ^ rs.r1_c2;
-  const float2 wd2 = make_float2(k.wd, k.wd), mu2 = make_float2(k.mu, k.mu);
-  const float2 neg_lr2 = make_float2(k.neg_lr, k.neg_lr);
+#pragma unroll 1
   for (int e = 0; e < rs.steps; ++e) {
-    const uint32_t c0_first = rs.r1_c0 ^ (rs.base_lo + (uint32_t)e);
-    uint32_t x[NB][4];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      x[b][0] = c0_first; x[b][1] = rs.r1_c1; x[b][2] = c2_first[b]; x[b][3] = gp.lo[b];
-    }
-#pragma unroll
-    for (int r = 1; r < 10; ++r)
-#pragma unroll
-      for (int b = 0; b < NB; ++b) philox_round(x[b][0], x[b][1], x[b][2], x[b][3], keys.a[r], keys.b[r]);
-    float2 r2[NB];  // squared radii of the block's two pairs
-    uint32_t top = 0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      r2[b] = Gen::radius2_pair(x[b][0], x[b][2], k.lg_scale);
-      top = max(top, max(x[b][0], x[b][2]));
-    }
-    if (Gen::needs_series(top)) {  // about once in 250 steps of a pack
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        if (Gen::needs_series(x[b][0])) r2[b].x = r2_next_to_one(x[b][0], k.scale2);
-        if (Gen::needs_series(x[b][2])) r2[b].y = r2_next_to_one(x[b][2], k.scale2);
-      }
-    }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const float2 theta = Gen::angle_pair(x[b][1], x[b][3]);
-      const float2 n01 = Gen::finish_pair(r2[b].x, theta.x);  // grad_std * (z0, z1)
-      const float2 n23 = Gen::finish_pair(r2[b].y, theta.y);  // grad_std * (z2, z3)
-      sgd_update_pair(w[4 * b], w[4 * b + 1], m[4 * b], m[4 * b + 1], n01, wd2, mu2, neg_lr2);
-      sgd_update_pair(w[4 * b + 2], w[4 * b + 3], m[4 * b + 2], m[4 * b + 3], n23, wd2, mu2, neg_lr2);
-    }
+    float2 nz[NB][2];
+    step_noise<Gen, NB>(nz, e, c2_first, gp, rs, keys, k);
+    step_update<NB>(w, m, nz, k);
   }
 }
 
@@ -1161,13 +1208,12 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
         // butterfly over the half-warp finishes the two sums.
         __syncthreads();
         for (int j = a.k - 1 + warp; j < a.n; j += kWarps) {
-          float v = 0.f;
+          double d = 0.0;
 #pragma unroll
           for (int wi = 0; wi < kWarps; ++wi) {
-            v += s_acc[j * kThreads + wi * 32 + lane];
+            d += (double)s_acc[j * kThreads + wi * 32 + lane];
             s_acc[j * kThreads + wi * 32 + lane] = 0.f;
           }
-          double d = (double)v;
 #pragma unroll
           for (int off = 8; off > 0; off >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, off);
           if ((lane & 15) == 0) s_part[r][2 * j + (lane >> 4)] += d;  // value = 2 * visit index + which
@@ -1413,6 +1459,407 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
     float *out_r = scratch.out_rounds + r * 2 * kMaxDevices;
     if (access_ok(out_r + at, 4)) out_r[at] = (float)sum;
     if (r + 1 == n_rounds && access_ok(scratch.out + at, 4)) scratch.out[at] = (float)sum;
+  });
+}
+
+// ------------------------------------------------------------------------------------------
+// Several rounds per launch with the replicas on the SM ("resident" batch).  A block of 128 threads takes
+// its columns through all rounds of the batch.  The rows are read from HBM once, live on the SM in between
+// and are written back once: parameters in shared memory, momentum in tensor memory - 256 KB per SM
+// that no kernel here needs for a contraction and that doubles what an SM can hold.  Rows that find no
+// room stay in the arena, i.e. in L2.  Either way a value is only ever touched by the thread that owns its
+// column, so no barrier separates the rows or rounds of a block.
+// The arithmetic of a round is that of k_round, in the same order: same results bit for bit.
+//
+// What bounds it: on large vectors the row walk through L2 ran into the board's power cap (1000 W, SM clock
+// down to 1600 - 1750 MHz); here a round moves a fraction of the bytes, keeps the full clock at 500 - 900 W
+// and is bound by instruction latency at 3 to 6 warps per scheduler (232 instructions per row and pack).
+// How many blocks share an SM decides between warps to hide latency with and rows that find room (the
+// host chooses).  Sustained, us per round of a batch of 8, row walk -> resident: 16 devices, 2^24, one
+// step 496 -> 430 (3, 4, 5, 6 blocks: 424, 436, 431, 478), two steps at 14.7 M 635 -> 534 (574, 556, 534,
+// 525); 8 devices, 11.2 M, one step 148 -> 125; 32 devices, 23.5 M 1955 -> 1599 (2, 3 blocks: 1830, 1599);
+// bf16 parameters, 16 devices, 2^22 125 -> 108; 16 devices, 14.7 M, steps 1,1,2,2,4,4,8,8: 863 (one launch
+// per round) -> 822 (3 .. 6 blocks: 935, 887, 844, 821).
+// A round that overwrites all devices stores the aggregate and reads nothing: all rows share its norm (16
+// devices, 12.8 M, steps 1,1,2,2,4,4,8,8, every round synchronised: 781 us per round with a read of every row
+// before its store, 677 without; one launch per round 748).
+// The first step's noise is drawn while the row's values are on their way (434 -> 421 us with everything on
+// the SM, 16 devices).  Each row is either wholly on the SM or wholly in the arena and the code is compiled
+// for either place: choosing at every access cost 100 instructions per row and pack in register copies.
+// ------------------------------------------------------------------------------------------
+constexpr int kResidentThreads = 128;
+constexpr int kResidentMaxBlocks = 6;  // per SM, by registers (80 a thread); shared memory sets the actual number
+
+struct ResidentBatch {
+  int32_t n, k, n_rounds;
+  int32_t n_on_chip;  // devices 0 .. n_on_chip - 1 live on the SM, the others in the arena
+  float beta, one_minus_beta;
+  int32_t write_all[kRoundBatchMax];                // as in RoundArgs
+  int32_t n_stepping[kRoundBatchMax];               // devices that run at least one step ...
+  int32_t order[kRoundBatchMax][kMaxDevices];       // ... by descending step count
+  int32_t draw[kRoundBatchMax][kMaxDevices];        // devices: the selected ones in draw order, then the rest
+  float a[kRoundBatchMax][kMaxDevices];             // aggregation weights in draw order
+  uint32_t r1_c0[kMaxDevices], r1_c1[kMaxDevices];  // as in RowStep
+  int64_t w_off[kMaxDevices], m_off[kMaxDevices];   // as in RowStep
+  RowsStep s[kRoundBatchMax][kMaxDevices];          // (visit is not used)
+};
+
+// A thread's packs in shared memory: [row][plane of 16 bytes][thread].
+template <typename WT>
+struct RowStore {
+  static constexpr int kPackBytes = 8 * (int)sizeof(WT);
+  static constexpr int kPlanes = kPackBytes / 16;
+  static constexpr int kRowBytes = kPackBytes * kResidentThreads;
+  static __device__ __forceinline__ void load(const char *mine, int row, RawPack<WT, 8> &r) {
+    uint4 u[kPlanes];
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i)
+      u[i] = *reinterpret_cast<const uint4 *>(mine + row * kRowBytes + i * 16 * kResidentThreads);
+    memcpy(&r, u, kPackBytes);
+  }
+  static __device__ __forceinline__ void store(char *mine, int row, const RawPack<WT, 8> &r) {
+    uint4 u[kPlanes];
+    memcpy(u, &r, kPackBytes);
+#pragma unroll
+    for (int i = 0; i < kPlanes; ++i)
+      *reinterpret_cast<uint4 *>(mine + row * kRowBytes + i * 16 * kResidentThreads) = u[i];
+  }
+};
+
+// Tensor memory as per-thread storage: a warp owns the 32 lanes of its quarter, a thread one lane; a pack
+// is 4 or 8 consecutive 32-bit columns of that lane.  A load is complete after tmem_wait_load (the values
+// pass through tmem_use there, so that nothing reads them before), a store is visible to the thread's
+// later loads after tmem_wait_store.
+__device__ __forceinline__ void tmem_load(uint32_t at, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(at));
+}
+__device__ __forceinline__ void tmem_load(uint32_t at, uint32_t (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
+}
+__device__ __forceinline__ void tmem_store(uint32_t at, const uint32_t (&v)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(at), "r"(v[0]), "r"(v[1]),
+               "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+__device__ __forceinline__ void tmem_store(uint32_t at, const uint32_t (&v)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_load() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_store() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void tmem_use(uint32_t (&v)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(v[i]));
+}
+
+// Columns of tensor memory that hold n packs of `words` words: a power of two, 32 at least.
+__host__ __device__ constexpr int tmem_columns(int n, int words) {
+  int c = 32;
+  while (c < n * words) c *= 2;
+  return c;
+}
+
+// Row sums of a warp that no other warp takes part in: the fp32 part of the order is k_round's (a
+// thread's pack, then the lanes l and l ^ 16), the rest is added in fp64, as there.  add() leaves 32 values
+// per row in the warp's slots, fold() adds those of up to 4 rows: 8 lanes per row.
+struct WarpRowSums {
+  static constexpr int kRows = 4;
+  static constexpr int kFloats = kRows * 32;
+  static __device__ __forceinline__ void add(float *slots, int s, float n2, float d2, int lane) {
+    const bool upper = (lane & 16) != 0;
+    const float keep = upper ? d2 : n2, give = upper ? n2 : d2;
+    slots[s * 32 + lane] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, 16);
+  }
+  // sums of the visit indices j0 .. j0 + count - 1 -> line[2 j + which]
+  static __device__ __forceinline__ void fold(const float *slots, int j0, int count, double *line, int lane) {
+    __syncwarp();
+    const float4 v = reinterpret_cast<const float4 *>(slots)[lane];
+    double d = ((double)v.x + (double)v.y) + ((double)v.z + (double)v.w);
+    d += __shfl_xor_sync(0xFFFFFFFFu, d, 1);
+    d += __shfl_xor_sync(0xFFFFFFFFu, d, 2);
+    if ((lane & 3) == 0 && (lane >> 3) < count) line[2 * j0 + (lane >> 2)] = d;
+    __syncwarp();
+  }
+};
+
+// Shared memory of a block beside its rows: [warp][round][2 n] sums and the warps' slots.
+constexpr size_t resident_sums_bytes(int n, int rounds) {
+  return (kResidentThreads / 32) * (sizeof(double) * 2 * n * rounds + sizeof(float) * WarpRowSums::kFloats);
+}
+
+template <typename WT, typename MT, typename Gen, int RM, bool kAllOnChip>
+__global__ void __launch_bounds__(kResidentThreads, kResidentMaxBlocks)
+k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, PhiloxKeys keys,
+                  StepConsts k, RoundScratch scratch, const __grid_constant__ ResidentBatch b) {
+  constexpr int E = 8, kWarps = kResidentThreads / 32;
+  constexpr int kWords = E * (int)sizeof(MT) / 4;  // tensor memory columns per row
+  using Store = RowStore<WT>;
+  using Sums = WarpRowSums;
+  extern __shared__ __align__(16) char s_raw[];
+  __shared__ uint32_t s_tmem;
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = b.n, n_sel = b.k, n_on_chip = kAllOnChip ? n : b.n_on_chip;
+  const int n_vals = b.n_rounds * 2 * n;
+  char *mine = s_raw + 16 * threadIdx.x;                                        // [row][plane][thread]
+  double *lines = reinterpret_cast<double *>(s_raw + n_on_chip * Store::kRowBytes);  // [warp][round][2 n]
+  float *slots = reinterpret_cast<float *>(lines + kWarps * n_vals) + warp * Sums::kFloats;
+
+  const int cols = tmem_columns(n_on_chip, kWords);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(&s_tmem)), "r"(cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tm = s_tmem + ((uint32_t)warp << 21);  // this warp's quarter: lanes 32 * warp ...
+
+  const int64_t n_packs = (n_params + E - 1) / E;
+  const int64_t n_chunks = (n_packs + kResidentThreads - 1) / kResidentThreads;
+  for (int64_t chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
+    auto do_chunk = [&](auto all_full) {
+      const int64_t p = chunk * kResidentThreads + threadIdx.x;
+      const int live = decltype(all_full)::value ? E : live_of(n_params, p, E);
+      const GroupProducts<E / 4> gp(p);
+      char *wp = reinterpret_cast<char *>(w) + p * (int64_t)(E * sizeof(WT));
+      char *mp = reinterpret_cast<char *>(m) + p * (int64_t)(E * sizeof(MT));
+      // A row's packs where they live; `where` is std::true_type for the SM, std::false_type for the arena.
+      auto load_w = [&](auto where, int row, RawPack<WT, E> &r) {
+        if constexpr (decltype(where)::value)
+          Store::load(mine, row, r);
+        else
+          ld_raw(at_row<WT>(wp, b.w_off[row]), live, r);
+      };
+      auto store_w = [&](auto where, int row, const RawPack<WT, E> &r) {
+        if constexpr (decltype(where)::value)
+          Store::store(mine, row, r);
+        else
+          st_raw(at_row<WT>(wp, b.w_off[row]), live, r);
+      };
+      auto load_m = [&](auto where, int row, RawPack<MT, E> &r) {  // the values: through m_values
+        if constexpr (decltype(where)::value) {
+          uint32_t v[kWords];
+          tmem_load(tm + row * kWords, v);
+          memcpy(&r, v, sizeof(v));
+        } else {
+          ld_raw(at_row<MT>(mp, b.m_off[row]), live, r);
+        }
+      };
+      auto m_values = [&](auto where, RawPack<MT, E> &r, float (&mv)[E]) {
+        if constexpr (decltype(where)::value) {
+          uint32_t v[kWords];
+          tmem_wait_load();
+          memcpy(v, &r, sizeof(v));
+          tmem_use(v);
+          memcpy(&r, v, sizeof(v));
+        }
+        unpack(r, mv);
+      };
+      auto store_m = [&](auto where, int row, const float (&mv)[E]) {
+        RawPack<MT, E> r;
+        pack_raw(mv, r);
+        if constexpr (decltype(where)::value) {
+          uint32_t v[kWords];
+          memcpy(v, &r, sizeof(v));
+          tmem_store(tm + row * kWords, v);
+        } else {
+          st_raw(at_row<MT>(mp, b.m_off[row]), live, r);
+        }
+      };
+      // A row's parameters as they stand, dead lanes 0.
+      auto values = [&](auto where, int row, float (&wv)[E]) {
+        RawPack<WT, E> r;
+        load_w(where, row, r);
+        unpack(r, wv);
+        if (live < E) {
+#pragma unroll
+          for (int i = 0; i < E; ++i) wv[i] = i < live ? wv[i] : 0.f;
+        }
+      };
+      // f for a row, compiled for either place (a choice at every access costs copies of the registers)
+      auto at_place = [&](int row, auto f) {
+        if (kAllOnChip || row < n_on_chip)
+          f(std::true_type{}, row);
+        else if constexpr (!kAllOnChip)
+          f(std::false_type{}, row);
+      };
+
+      // ---- the rows come in
+#pragma unroll 1
+      for (int row = 0; row < n_on_chip; ++row) {
+        RawPack<WT, E> rw;
+        RawPack<MT, E> rm;
+        float mv[E];
+        ld_raw(at_row<WT>(wp, b.w_off[row]), live, rw);
+        load_m(std::false_type{}, row, rm);
+        m_values(std::false_type{}, rm, mv);
+        store_w(std::true_type{}, row, rw);
+        store_m(std::true_type{}, row, mv);
+      }
+      tmem_wait_store();
+
+#pragma unroll 1
+      for (int r = 0; r < b.n_rounds; ++r) {
+        double *line = lines + (warp * b.n_rounds + r) * 2 * n;
+        // ---- local steps
+        const int n_step = b.n_stepping[r];
+#pragma unroll 1
+        for (int j = 0; j < n_step; ++j) {
+          const int row = b.order[r][j];
+          RowStep rs;
+          rs.row = row;
+          rs.steps = b.s[r][row].steps;
+          rs.base_lo = b.s[r][row].base_lo;
+          rs.r1_c2 = b.s[r][row].r1_c2;
+          rs.r1_c0 = b.r1_c0[row];
+          rs.r1_c1 = b.r1_c1[row];
+          uint32_t c2_first[E / 4];
+#pragma unroll
+          for (int g = 0; g < E / 4; ++g) c2_first[g] = gp.hi[g] ^ rs.r1_c2;
+          at_place(row, [&](auto where, int row) {
+            float wv[E], mv[E];
+            RawPack<WT, E> rw;
+            RawPack<MT, E> rm;
+            load_m(where, row, rm);
+            load_w(where, row, rw);
+            // the values are on their way while the first step's noise is drawn
+            float2 nz[E / 4][2];
+            step_noise<Gen, E / 4>(nz, 0, c2_first, gp, rs, keys, k);
+            m_values(where, rm, mv);
+            unpack(rw, wv);
+            step_update<E / 4>(wv, mv, nz, k);
+#pragma unroll 1
+            for (int e = 1; e < rs.steps; ++e) {
+              step_noise<Gen, E / 4>(nz, e, c2_first, gp, rs, keys, k);
+              step_update<E / 4>(wv, mv, nz, k);
+            }
+            if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, rs, keys);
+            pack_raw(wv, rw);
+            store_w(where, row, rw);
+            store_m(where, row, mv);
+          });
+        }
+        // ---- aggregation with write-back: acc = a_0 w_0, then acc = fma(a_j, w_j, acc) in draw order
+        float acc[E];
+        at_place(b.draw[r][0], [&](auto where, int row) {
+          float wv[E];
+          values(where, row, wv);
+          const float a0 = b.a[r][0];
+#pragma unroll
+          for (int i = 0; i < E; ++i) acc[i] = __fmul_rn(a0, wv[i]);
+        });
+#pragma unroll 1
+        for (int j = 1; j < n_sel; ++j)
+          at_place(b.draw[r][j], [&](auto where, int row) {
+            float wv[E];
+            values(where, row, wv);
+            const float aj = b.a[r][j];
+#pragma unroll
+            for (int i = 0; i < E; ++i) acc[i] = fmaf(aj, wv[i], acc[i]);
+          });
+        float n2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          acc[i] = as_stored(acc[i], w);
+          n2 = fmaf(acc[i], acc[i], n2);
+        }
+        const int write_all = b.write_all[r], n_holders = write_all == 1 ? n : n_sel;
+        {
+          RawPack<WT, E> ra;
+          pack_raw(acc, ra);
+#pragma unroll 1
+          for (int t = 0; t < n_holders; ++t)
+            at_place(b.draw[r][t], [&](auto where, int row) { store_w(where, row, ra); });
+        }
+        Sums::add(slots, 0, n2, 0.f, lane);  // one value for all holders
+        // ---- the other devices: keep their own model, or mix the aggregate into it
+        int slot = 0;
+#pragma unroll 1
+        for (int j = n_holders; j < n; ++j) {
+          float s2 = 0.f, d2 = 0.f;
+          at_place(b.draw[r][j], [&](auto where, int row) {
+            float wv[E];
+            values(where, row, wv);
+            if (write_all) {
+#pragma unroll
+              for (int i = 0; i < E; ++i)
+                wv[i] = as_stored(fmaf(b.beta, acc[i], __fmul_rn(b.one_minus_beta, wv[i])), w);
+              RawPack<WT, E> rw;
+              pack_raw(wv, rw);
+              store_w(where, row, rw);
+            }
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+              const float d = wv[i] - acc[i];
+              s2 = fmaf(wv[i], wv[i], s2);
+              d2 = fmaf(d, d, d2);
+            }
+          });
+          if (++slot == Sums::kRows) {
+            Sums::fold(slots, j - Sums::kRows, Sums::kRows, line, lane);
+            slot = 0;
+          }
+          Sums::add(slots, slot, s2, d2, lane);
+        }
+        Sums::fold(slots, write_all == 1 ? n_sel - 1 : n - 1 - slot, slot + 1, line, lane);
+        tmem_wait_store();
+      }
+
+      // ---- the rows go back
+#pragma unroll 1
+      for (int row = 0; row < n_on_chip; ++row) {
+        RawPack<WT, E> rw;
+        RawPack<MT, E> rm;
+        float mv[E];
+        load_m(std::true_type{}, row, rm);
+        load_w(std::true_type{}, row, rw);
+        m_values(std::true_type{}, rm, mv);
+        st_raw(at_row<WT>(wp, b.w_off[row]), live, rw);
+        store_m(std::false_type{}, row, mv);
+      }
+    };
+    if ((chunk + 1) * kResidentThreads * E <= n_params)
+      do_chunk(std::true_type{});
+    else
+      do_chunk(std::false_type{});
+    // devices that hold the aggregate share one sum
+    auto has_sum = [&](int t) {
+      const int r = t / (2 * n), j = (t - r * 2 * n) >> 1;
+      return j >= n_sel - 1 && (j < n_sel || b.write_all[r] != 1);
+    };
+    __syncthreads();
+    for (int t = threadIdx.x; t < n_vals; t += kResidentThreads) {  // a value belongs to one thread
+      double *at = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
+      double sum = chunk == blockIdx.x ? 0.0 : *at;
+      if (has_sum(t))
+        for (int wi = 0; wi < kWarps; ++wi) sum += lines[wi * n_vals + t];
+      if (access_ok(at, 8)) *at = sum;
+    }
+    __syncthreads();
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(cols));
+
+  finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
+                   [&](int t, double sum) {
+    const int r = t / (2 * n), v = t - r * 2 * n, j = v >> 1, which = v & 1;
+    float *out_r = scratch.out_rounds + r * 2 * kMaxDevices;
+    auto put = [&](int at, float x) {
+      if (access_ok(out_r + at, 4)) out_r[at] = x;
+      if (r + 1 == b.n_rounds && access_ok(scratch.out + at, 4)) scratch.out[at] = x;
+    };
+    if (j == n_sel - 1) {  // the holders of the aggregate share one norm and are at distance 0
+      for (int q = 0; q < (b.write_all[r] == 1 ? n : n_sel); ++q) put(which * n + b.draw[r][q], which ? 0.f : (float)sum);
+    } else if (j >= n_sel && b.write_all[r] != 1) {
+      put(which * n + b.draw[r][j], (float)sum);
+    }
   });
 }
 

@@ -1,0 +1,68 @@
+"""Batches of rounds whose replicas stay on the SMs (shared memory and tensor memory) against the same rounds
+launched one by one, bit for bit: arenas beyond the L2 with all rows on the SM (few devices), with part of
+them (16 devices and more), light and heavy steps, every storage, ragged ends, odd numbers of rounds,
+global synchronisation by overwriting and by mixing, devices that run no steps, one and all devices
+selected; and small arenas of at most 8 devices, which take the form as well.  The statistics' fp64 sums
+are added in another order: equal to one rounding of the fp32 output."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_common import require_gpu
+from paper_2111_08274_b200 import runtime, workloads
+from paper_2111_08274_b200.workloads import Workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+STORAGE = {"fp32": (0, 0, 0, 8), "bf16": (1, 0, 0, 6), "bf16_m16": (1, 1, 0, 4), "bf16_m16_sr": (1, 1, 1, 4)}
+
+
+def compare(n, P, k, steps, storage, beta, batches, launches):
+    dtype, m_dtype, rounding, _ = STORAGE[storage]
+    rounds = sum(batches)
+    wl = Workload("res", n, P, k, rounds, "fixed", steps, grad_std=1e-2, dtype=dtype, m_dtype=m_dtype, rounding=rounding,
+                  sync_every=3, sync_beta=beta, seed=workloads.BASE_SEED + P + n)
+    batch, single = runtime.Arena(wl), runtime.Arena(wl)
+    single.h.set_round_batch(1)
+    for a in (batch, single):                     # what lies behind the vector must stay as it is
+        a.w[:, P:] = 3.0
+        a.m[:, P:] = 5.0
+    before, first, got = batch.h.launch_count(), 0, []
+    for count in batches:
+        got.append(batch.run_rounds_fused(first, count))
+        first += count
+    assert batch.h.launch_count() - before == launches
+    want = single.run_rounds_fused(0, rounds)
+    assert np.array_equal(np.concatenate(got), want)
+    torch.cuda.synchronize()
+    assert torch.equal(batch.w, single.w) and torch.equal(batch.m, single.m)
+    va, vb = batch.h.get_versions(), single.h.get_versions()
+    assert np.array_equal(va[0], vb[0]) and np.array_equal(va[1], vb[1])
+    a, b = batch.h.stats_read(), single.h.stats_read()
+    assert np.allclose(a[0], b[0], rtol=2.0 ** -23, atol=0) and np.allclose(a[1], b[1], rtol=2.0 ** -23, atol=0)
+    batch.h.debug_check()
+    batch.close()
+    single.close()
+
+
+@pytest.mark.parametrize("storage", sorted(STORAGE))
+@pytest.mark.parametrize("n,k,hi", [(2, 1, 2), (5, 5, 2), (8, 4, 2), (8, 3, 7), (13, 2, 2), (16, 4, 2), (16, 16, 5), (24, 3, 2),
+                                    (32, 8, 2)])
+def test_large_arenas(n, k, hi, storage):
+    rounding = STORAGE[storage][2]
+    P = 150_000_001 // (n * STORAGE[storage][3]) // 1024 * 1024 + {2: 1, 5: 1023, 8: 8, 13: 519}.get(n, 0)
+    steps = tuple((3 * i + 1) % (hi + 1) for i in range(n))
+    compare(n, P, k, steps, storage, 0.25 if n % 2 else 1.0, (8, 3, 1),
+            12 if rounding and n > 16 else 3)   # stochastic rounding with many devices: one by one
+
+
+@pytest.mark.parametrize("n,P,k", [(8, 524_289, 4), (3, 1_500_007, 2), (1, 4_200_001, 1), (8, 1_048_576, 8)])
+@pytest.mark.parametrize("hi", [1, 6])
+def test_small_arenas(n, P, k, hi):
+    compare(n, P, k, tuple((3 * i + 1) % (hi + 1) for i in range(n)), "fp32", 0.5, (2, 7), 2)
