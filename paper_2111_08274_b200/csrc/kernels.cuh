@@ -231,6 +231,43 @@ __device__ __forceinline__ void st_pack_any(T *row, int64_t p, int live, const f
       if (i < live) st_elem(row, E * p + i, v[i]);
   }
 }
+// Full packs (`live` is a compile-time E) of an arena whose rows start at multiples of 32 bytes: 8 fp32 values
+// in one 32-byte store.  Two 16-byte stores of a warp cover half of each sector, and where L1 does not hold
+// the line they reach L2 as two partial writes (30 % more write sectors in a batch that overwrites all
+// devices).  Measured, us, two stores / one: resident batches, 16 devices, 2^24, one step 428 / 405 per round,
+// 32 devices, 23.5 M 1602 / 1572; fused round, 8 devices, 11.2 M, one step 238.7 / 232.4; 16 devices, 2^25,
+// one step 1300 / 1292.  A test of the address at each store cost what it gave (8 steps 578 -> 584 .. 588),
+// hence the compile-time choice.  32-byte loads gain nothing (the line stays in L1 between the two halves)
+// and cost bf16 rounds of 8 steps 2 %.
+__device__ __forceinline__ void st_full(float *at, const float (&v)[8]) {
+  if (!access_ok(at, 32)) return;
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(at), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+               "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+}
+template <int E>
+struct FullPack {  // a number of live lanes that is E at compile time
+  __device__ constexpr operator int() const { return E; }
+};
+template <typename T, int E>
+__device__ __forceinline__ void st_pack_any(T *row, int64_t p, FullPack<E>, const float (&v)[E]) {
+  if constexpr (sizeof(T) == 4 && E == 8)
+    st_full(row + E * p, v);
+  else
+    st_pack<E>(row, p, v);
+}
+template <typename T>
+__device__ __forceinline__ void st_raw(T *at, FullPack<8>, const RawPack<T, 8> &r) {
+  if constexpr (sizeof(T) == 4)
+    st_full(at, r.v);
+  else
+    st_raw(at, 8, r);
+}
+// Whether the fp32 rows behind w and m (their distance is a multiple of 32 bytes) start at multiples of 32.
+template <typename WT, typename MT>
+__device__ __forceinline__ bool rows_at_32(const WT *w, const MT *m) {
+  const uintptr_t at = (sizeof(WT) == 4 ? (uintptr_t)w : 0) | (sizeof(MT) == 4 ? (uintptr_t)m : 0);
+  return (at & 31) == 0;
+}
 // The value a parameter has once stored: itself for fp32, rounded to nearest even for bf16.
 __device__ __forceinline__ float as_stored(float v, const float *) { return v; }
 __device__ __forceinline__ float as_stored(float v, const __nv_bfloat16 *) {
@@ -239,6 +276,14 @@ __device__ __forceinline__ float as_stored(float v, const __nv_bfloat16 *) {
 __device__ __forceinline__ int live_of(int64_t n_params, int64_t p, int E) {
   const int64_t left = n_params - (int64_t)E * p;
   return left >= E ? E : (left > 0 ? (int)left : 0);
+}
+template <int E>
+__device__ __forceinline__ FullPack<E> live_of(std::true_type, int64_t, int64_t) {
+  return {};
+}
+template <int E>
+__device__ __forceinline__ int live_of(std::false_type, int64_t n_params, int64_t p) {
+  return live_of(n_params, p, E);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -581,9 +626,10 @@ k_local_step(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, LocalStep
   const int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   // The body is compiled twice: for blocks whose packs are all full (`live` is then the constant
   // E and every ragged-tail test in the loads and stores folds away: 2-3 % fewer instructions per
-  // row) and for the one block that holds the end of the vector.
+  // row, and 32-byte stores) and for the one block that holds the end of the vector, or all blocks of an arena
+  // whose rows do not start at multiples of 32 bytes.
   auto run = [&](auto all_full) {
-    const int live = decltype(all_full)::value ? E : live_of(n_params, p, E);
+    const auto live = live_of<E>(all_full, n_params, p);
     if (live == 0) return;
     const GroupProducts<E / 4> gp(p);
     char *wp = reinterpret_cast<char *>(w) + p * (int64_t)(E * sizeof(WT));
@@ -629,7 +675,7 @@ k_local_step(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, LocalStep
       visit(j, rw, rm);
     }
   };
-  if (((int64_t)blockIdx.x + 1) * kThreads * E <= n_params)
+  if (((int64_t)blockIdx.x + 1) * kThreads * E <= n_params && rows_at_32(w, m))
     run(std::true_type{});
   else
     run(std::false_type{});
@@ -1099,11 +1145,12 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
   const int64_t n_chunks = (n_packs + kThreads - 1) / kThreads;
   for (int64_t chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
     // The chunk's work is compiled twice: for chunks whose packs are all full (`live` is then the
-    // constant E and every ragged-tail test in the loads and stores folds away) and for the chunk
-    // that holds the end of the vector (and, there, the lanes beyond it).
+    // constant E, every ragged-tail test in the loads and stores folds away and stores are of 32 bytes)
+    // and for the chunk that holds the end of the vector (and, there, the lanes beyond it), or all
+    // chunks of an arena whose rows do not start at multiples of 32 bytes.
     auto do_chunk = [&](auto all_full) {
       const int64_t p = chunk * kThreads + threadIdx.x;
-      const int live = decltype(all_full)::value ? E : live_of(n_params, p, E);
+      const auto live = live_of<E>(all_full, n_params, p);
       const GroupProducts<E / 4> gp(p);
       char *wp = reinterpret_cast<char *>(w) + p * (int64_t)(E * sizeof(WT));
       char *mp = reinterpret_cast<char *>(m) + p * (int64_t)(E * sizeof(MT));
@@ -1228,7 +1275,7 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
         for (int r = 0; r < b.n_rounds; ++r) do_round(b.round[r], r);
       }
     };
-    if ((chunk + 1) * kThreads * E <= n_params)
+    if ((chunk + 1) * kThreads * E <= n_params && rows_at_32(w, m))
       do_chunk(std::true_type{});
     else
       do_chunk(std::false_type{});
@@ -1351,7 +1398,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
   for (int64_t tile = (int64_t)blockIdx.x * groups + group; tile < n_tiles; tile += (int64_t)gridDim.x * groups) {
     auto do_tile = [&](auto all_full) {
       const int64_t p = tile * 32 + lane;
-      const int live = decltype(all_full)::value ? E : live_of(n_params, p, E);
+      const auto live = live_of<E>(all_full, n_params, p);
       const GroupProducts<E / 4> gp(p);
       WT *wp = w + row * stride + p * E;
       MT *mp = m + row * stride + p * E;
@@ -1440,7 +1487,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
       // the next tile's first round must not overwrite a buffer that is still being read
       asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(n * 32) : "memory");
     };
-    if ((tile + 1) * 32 * E <= n_params)
+    if ((tile + 1) * 32 * E <= n_params && rows_at_32(w, m))
       do_tile(std::true_type{});
     else
       do_tile(std::false_type{});
@@ -1476,8 +1523,8 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 // and is bound by instruction latency at 3 to 6 warps per scheduler (232 instructions per row and pack).
 // How many blocks share an SM decides between warps to hide latency with and rows that find room (the
 // host chooses).  Sustained, us per round of a batch of 8, row walk -> resident: 16 devices, 2^24, one
-// step 496 -> 430 (3, 4, 5, 6 blocks: 424, 436, 431, 478), two steps at 14.7 M 635 -> 534 (574, 556, 534,
-// 525); 8 devices, 11.2 M, one step 148 -> 125; 32 devices, 23.5 M 1955 -> 1599 (2, 3 blocks: 1830, 1599);
+// step 496 -> 409 (before the 32-byte stores 3, 4, 5, 6 blocks: 424, 436, 431, 478), two steps at 14.7 M 635 -> 534 (574, 556, 534,
+// 525); 8 devices, 11.2 M, one step 148 -> 124; 32 devices, 23.5 M 1955 -> 1574 (2, 3 blocks: 1830, 1599);
 // bf16 parameters, 16 devices, 2^22 125 -> 108; 16 devices, 14.7 M, steps 1,1,2,2,4,4,8,8: 863 (one launch
 // per round) -> 822 (3 .. 6 blocks: 935, 887, 844, 821).
 // A round that overwrites all devices stores the aggregate and reads nothing: all rows share its norm (16
@@ -1624,7 +1671,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
   for (int64_t chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
     auto do_chunk = [&](auto all_full) {
       const int64_t p = chunk * kResidentThreads + threadIdx.x;
-      const int live = decltype(all_full)::value ? E : live_of(n_params, p, E);
+      const auto live = live_of<E>(all_full, n_params, p);
       const GroupProducts<E / 4> gp(p);
       char *wp = reinterpret_cast<char *>(w) + p * (int64_t)(E * sizeof(WT));
       char *mp = reinterpret_cast<char *>(m) + p * (int64_t)(E * sizeof(MT));
@@ -1823,7 +1870,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
         store_m(std::false_type{}, row, mv);
       }
     };
-    if ((chunk + 1) * kResidentThreads * E <= n_params)
+    if ((chunk + 1) * kResidentThreads * E <= n_params && rows_at_32(w, m))
       do_chunk(std::true_type{});
     else
       do_chunk(std::false_type{});
