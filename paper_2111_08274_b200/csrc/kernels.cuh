@@ -1911,6 +1911,25 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
 }
 
 // ------------------------------------------------------------------------------------------
+// Backup snapshot of a bf16 row, widened to fp32.  Bound by memory (6 bytes per parameter), and small beside
+// the transfer that follows it.  dst is an allocation's start.
+// ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kThreads)
+k_widen(const __nv_bfloat16 *__restrict__ src, float *__restrict__ dst, int64_t count) {
+  const int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const int live = live_of(count, p, 8);
+  if (live == 0) return;
+  RawPack<__nv_bfloat16, 8> r;
+  float v[8];
+  ld_raw(src + 8 * p, live, r);
+  unpack(r, v);
+  if (live == 8)
+    st_pack_any(dst, p, FullPack<8>{}, v);
+  else
+    st_pack_any(dst, p, live, v);
+}
+
+// ------------------------------------------------------------------------------------------
 // Generator diagnostics.
 // ------------------------------------------------------------------------------------------
 __global__ void k_debug_philox(const uint32_t *__restrict__ ctr, PhiloxKeys keys, int64_t n,

@@ -408,6 +408,24 @@ def test_state_errors():
     assert list(h.get_versions()[1]) == [2**56 - 1, 1]
 
 
+@pytest.mark.parametrize("m_dtype", [0, 1])
+@pytest.mark.parametrize("count", [1, 7, 8, 9, 2047, 2048, 2049, 300_003])
+def test_backup_widens_bf16_on_the_device(count, m_dtype):
+    """Edges of the widening kernel's packs and blocks: the values that read_params widens on the host, and
+    nothing behind them."""
+    wl = small(3, 300_003, dtype=1, m_dtype=m_dtype)
+    h = gpu(wl)
+    values = np.random.default_rng(count).standard_normal(wl.n_params).astype(np.float32)
+    values[:6] = [0.0, -0.0, np.inf, -np.inf, 1e-39, -3e38]
+    h.write_params(2, values)
+    buf = torch.full((count + 8,), 5.0).pin_memory()
+    h.backup_begin(2, buf, count=count)
+    h.backup_wait()
+    assert np.array_equal(buf.numpy()[:count].view(np.uint32), h.read_params(2, count=count).view(np.uint32))
+    assert (buf.numpy()[count:] == 5.0).all()
+    h.debug_check()
+
+
 @pytest.mark.parametrize("dtype", [0, 1])
 def test_overlapped_backup_is_a_snapshot(dtype):
     """hadfl_backup_begin captures the row as it is at that point of the stream, even though later
