@@ -17,6 +17,8 @@
 
 using namespace hadfl;
 
+constexpr int kStatsWatch = 4;  // one call of 32 rounds, or a few rounds as separate calls
+
 struct hadfl_handle {
   hadfl_config cfg;
   int64_t stride = 0;
@@ -36,11 +38,15 @@ struct hadfl_handle {
   // K3 scratch
   double *d_partials = nullptr;
   unsigned int *d_ticket = nullptr;
-  // Statistics, in page-locked host memory that the kernels write: 2 N floats of the last round, then those of
-  // each round of a batch.  Reading them is a wait for the stream and no copy (a watched round of 4 devices
-  // and 100,000 parameters: 43.5 -> 31.6 us).
-  float *stats_out = nullptr;
-  float *round_stats_out = nullptr;  // [round of a batch][2 * kMaxDevices]
+  // Statistics: 2 * kMaxDevices floats of the last round, then as many of each round of a batch; one such buffer
+  // in device memory and one in page-locked host memory.  While statistics are being read - within the last
+  // kStatsWatch launches that made any - launches write to the host (reading is then a wait for the stream and
+  // no copy: a watched round of 4 devices and 100,000 parameters 43.5 -> 31 us), else to the device: stores
+  // to the host make the end of a launch 1 to 2 us later (6 devices, 150,001 parameters: 10.6 against 12.4 us).
+  float *stats_dev = nullptr, *stats_host = nullptr;
+  float *stats_at = nullptr;        // where the last launch with statistics wrote those of its (last) round
+  float *round_stats_at = nullptr;  // ... and the last launch of the fused round kernel those of each round
+  int stats_unread = kStatsWatch;   // launches with statistics since the last read
   int stats_lanes = 0;  // blocks per row of the statistics kernel
   bool stats_valid = false;
   // fused round kernel scratch
@@ -96,6 +102,7 @@ constexpr size_t kBatchSmallArenaBytes = (size_t)64 << 20;  // arenas up to this
 constexpr int kRowPerBlockMaxSteps = 2;  // up to this many steps per device a launch is memory-bound: the local update
                                          // then takes one row per block (fp32), the fused round prefetches rows (bf16)
 constexpr size_t kSmemReserve = 1024 + 64;  // per block: what the system takes, and the kernel's own variables
+constexpr size_t kStatsFloats = 2 * kMaxDevices;  // statistics of one round
 constexpr int kStatsU = 4;  // 16-byte packs per thread and chunk in the statistics kernel
 constexpr int64_t kRowsGridCap = 4096;         // most blocks of a fused-round launch with a warp per row
 constexpr int64_t kRoundGridCap = 16384;  // most blocks of a fused-round launch (bounds its scratch: 8 MB)
@@ -209,6 +216,35 @@ struct DeviceGuard {
   }
 };
 
+// Where the next launch writes its statistics.
+float *next_stats(hadfl_handle *h) {
+  h->stats_at = h->stats_unread < kStatsWatch ? h->stats_host : h->stats_dev;
+  if (h->stats_unread < kStatsWatch) ++h->stats_unread;
+  return h->stats_at;
+}
+RoundScratch round_scratch(hadfl_handle *h) {
+  float *out = next_stats(h);
+  h->round_stats_at = out + kStatsFloats;
+  return RoundScratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket, h->round_stats_at, out};
+}
+
+// Waits for the stream and returns statistics at `at` in host memory.
+int fetch_stats(hadfl_handle *h, const float *at, const float **out) {
+  const float *host = h->stats_host;
+  const bool on_device = at < host || at >= host + kStatsFloats * (1 + kRoundBatchMax);
+  if (on_device) {
+    float *copy = h->stats_host + (at - h->stats_dev);
+    HADFL_CUDA(h, cudaMemcpyAsync(copy, at, sizeof(float) * 2 * (size_t)h->cfg.n_devices, cudaMemcpyDeviceToHost,
+                                  h->stream));
+    at = copy;
+  }
+  HADFL_CUDA(h, cudaStreamSynchronize(h->stream));
+  HADFL_DEBUG_RESULT();
+  h->stats_unread = 0;
+  *out = at;
+  return HADFL_OK;
+}
+
 // Page-locks 64 bytes per device once per process, so that the driver's pool of page-locked memory outlives
 // the handles: a handle's statistics then cost 1 us to allocate instead of 1 ms.  Nothing ever uses the bytes;
 // where this fails, handles are only slower to make.
@@ -321,8 +357,7 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
     }
     const int grid = (int)rows_grid(q.n, h->cfg.n_params);
     const size_t smem = rows_shared_bytes<WT, E>(q.groups, q.n, q.k, b.n_rounds);
-    const RoundScratch scratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket,
-                               h->round_stats_out, h->stats_out};
+    const RoundScratch scratch = round_scratch(h);
     auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR>;
     if (smem > 48 * 1024)  // more than 16 selected devices
       HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -417,8 +452,7 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
     if (smem < floor_bytes && blocks_per_sm < kResidentMaxBlocks) smem = floor_bytes;
     const int64_t chunks = (h->cfg.n_params + 8 * kResidentThreads - 1) / (8 * kResidentThreads);
     const int grid = (int)(chunks < kRoundGridCap ? chunks : kRoundGridCap);
-    const RoundScratch scratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket,
-                               h->round_stats_out, h->stats_out};
+    const RoundScratch scratch = round_scratch(h);
     auto kernel = q.n_on_chip == n ? k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, true>
                                    : k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, false>;
     HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -440,8 +474,7 @@ int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
     const size_t smem = sizeof(float) * kThreads * (size_t)h->cfg.n_devices;
     constexpr int E = StepPack<WT>::E;
     constexpr int RM = decltype(rm)::value;
-    const RoundScratch scratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket,
-                               h->round_stats_out, h->stats_out};
+    const RoundScratch scratch = round_scratch(h);
     int max_steps = 0;
     int64_t sum_steps = 0, n_rows = 0;
     for (int r = 0; r < b.n_rounds; ++r)
@@ -506,7 +539,7 @@ template <typename WT>
 int launch_stats(hadfl_handle *h, int ref) {
   k_stats<WT, kStatsU><<<h->stats_lanes * h->cfg.n_devices, kThreads, 0, h->stream>>>(
       (const WT *)h->w, h->stride, h->cfg.n_params, h->cfg.n_devices, ref, h->stats_lanes,
-      h->d_partials, h->d_ticket, h->stats_out);
+      h->d_partials, h->d_ticket, next_stats(h));
   return check_launch(h);
 }
 
@@ -627,11 +660,14 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_partials,
                            sizeof(double) * 2 * (size_t)cfg->n_devices * (size_t)lanes));
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_ticket, sizeof(unsigned int)));
-  const size_t stats_bytes = sizeof(float) * 2 * kMaxDevices;
+  const size_t stats_bytes = sizeof(float) * kStatsFloats * (1 + kRoundBatchMax);
   keep_host_pool(h->device);
-  HADFL_CUDA(h, cudaHostAlloc((void **)&h->stats_out, stats_bytes * (1 + kRoundBatchMax), cudaHostAllocMapped));
-  memset(h->stats_out, 0, stats_bytes * (1 + kRoundBatchMax));
-  h->round_stats_out = h->stats_out + 2 * kMaxDevices;
+  HADFL_CUDA(h, cudaMalloc((void **)&h->stats_dev, stats_bytes));
+  HADFL_CUDA(h, cudaMemsetAsync(h->stats_dev, 0, stats_bytes, h->stream));
+  HADFL_CUDA(h, cudaHostAlloc((void **)&h->stats_host, stats_bytes, cudaHostAllocMapped));
+  memset(h->stats_host, 0, stats_bytes);
+  h->stats_at = h->stats_dev;
+  h->round_stats_at = h->stats_dev + kStatsFloats;
   // Fused round kernel: one block per chunk of kThreads packs (8 columns each) up to kRoundGridCap
   // blocks, beyond which the blocks stride over the chunks.  Measured on the workloads' sizes, a grid
   // of many short blocks beats one resident wave by 7-15 % with several steps per device and is
@@ -673,10 +709,10 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
   debug_add(h->w, elems * elem_size(h));
   debug_add(h->m, elems * m_elem_size(h));
   debug_add(h->d_partials, sizeof(double) * 2 * (size_t)cfg->n_devices * (size_t)lanes);
-  debug_add(h->stats_out, stats_bytes);
+  debug_add(h->stats_dev, stats_bytes);
+  debug_add(h->stats_host, stats_bytes);
   debug_add(h->d_round_partials, sizeof(double) * round_vals * (size_t)scratch_grid);
   debug_add(h->d_round_group_partials, sizeof(double) * round_vals * n_groups);
-  debug_add(h->round_stats_out, stats_bytes * kRoundBatchMax);
   HADFL_CUDA(h, cudaDeviceSynchronize());
   if (debug_publish()) return HADFL_ERR_CUDA;
 #endif
@@ -694,10 +730,10 @@ int hadfl_destroy(hadfl_handle *h) {
   debug_remove(h->m);
   debug_remove(h->d_partials);
   debug_remove(h->d_backup);
-  debug_remove(h->stats_out);
+  debug_remove(h->stats_dev);
+  debug_remove(h->stats_host);
   debug_remove(h->d_round_partials);
   debug_remove(h->d_round_group_partials);
-  debug_remove(h->round_stats_out);
   debug_publish();
 #endif
   if (h->own_arena) {
@@ -706,7 +742,8 @@ int hadfl_destroy(hadfl_handle *h) {
   }
   cudaFree(h->d_partials);
   cudaFree(h->d_ticket);
-  cudaFreeHost(h->stats_out);
+  cudaFree(h->stats_dev);
+  cudaFreeHost(h->stats_host);
   cudaFree(h->d_round_partials);
   cudaFree(h->d_round_group_partials);
   cudaFree(h->d_round_ticket);
@@ -1107,9 +1144,9 @@ int hadfl_stats_read_round(hadfl_handle *h, int32_t back, float *out_norm2, floa
   if (!h->stats_valid || back >= h->last_launch_rounds) return HADFL_ERR_STATE;
   DeviceGuard guard(h->device);
   const int n = h->cfg.n_devices;
-  const float *src = h->round_stats_out + (size_t)(h->last_launch_rounds - 1 - back) * 2 * kMaxDevices;
-  HADFL_CUDA(h, cudaStreamSynchronize(h->stream));
-  HADFL_DEBUG_RESULT();
+  const float *src = nullptr;
+  const int rc = fetch_stats(h, h->round_stats_at + (size_t)(h->last_launch_rounds - 1 - back) * kStatsFloats, &src);
+  if (rc != HADFL_OK) return rc;
   memcpy(out_norm2, src, sizeof(float) * (size_t)n);
   memcpy(out_div2, src + n, sizeof(float) * (size_t)n);
   return HADFL_OK;
@@ -1129,10 +1166,11 @@ int hadfl_stats_read(hadfl_handle *h, float *out_norm2, float *out_div2) {
   if (!h->stats_valid) return HADFL_ERR_STATE;
   DeviceGuard guard(h->device);
   const int n = h->cfg.n_devices;
-  HADFL_CUDA(h, cudaStreamSynchronize(h->stream));
-  HADFL_DEBUG_RESULT();
-  memcpy(out_norm2, h->stats_out, sizeof(float) * (size_t)n);
-  memcpy(out_div2, h->stats_out + n, sizeof(float) * (size_t)n);
+  const float *src = nullptr;
+  const int rc = fetch_stats(h, h->stats_at, &src);
+  if (rc != HADFL_OK) return rc;
+  memcpy(out_norm2, src, sizeof(float) * (size_t)n);
+  memcpy(out_div2, src + n, sizeof(float) * (size_t)n);
   return HADFL_OK;
 }
 
