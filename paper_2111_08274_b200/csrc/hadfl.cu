@@ -216,16 +216,16 @@ struct DeviceGuard {
   }
 };
 
-// Where the next launch writes its statistics.
-float *next_stats(hadfl_handle *h) {
-  h->stats_at = h->stats_unread < kStatsWatch ? h->stats_host : h->stats_dev;
+// Where the next launch writes its statistics, and the note that it has been enqueued (a launch that failed leaves
+// the statistics of the one before it readable).
+float *next_stats(const hadfl_handle *h) { return h->stats_unread < kStatsWatch ? h->stats_host : h->stats_dev; }
+void stats_enqueued(hadfl_handle *h, float *out) {
+  h->stats_at = out;
   if (h->stats_unread < kStatsWatch) ++h->stats_unread;
-  return h->stats_at;
 }
-RoundScratch round_scratch(hadfl_handle *h) {
+RoundScratch round_scratch(const hadfl_handle *h) {
   float *out = next_stats(h);
-  h->round_stats_at = out + kStatsFloats;
-  return RoundScratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket, h->round_stats_at, out};
+  return RoundScratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket, out + kStatsFloats, out};
 }
 
 // Waits for the stream and returns statistics at `at` in host memory.
@@ -337,7 +337,7 @@ int64_t rows_grid(int n_devices, int64_t n_params) {
 }
 
 template <int NR>
-int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
+int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const RoundScratch &scratch) {
   return for_storage(h, [&](auto wt, auto mt, auto rm) {
     using WT = typename decltype(wt)::type;
     using MT = typename decltype(mt)::type;
@@ -357,7 +357,6 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
     }
     const int grid = (int)rows_grid(q.n, h->cfg.n_params);
     const size_t smem = rows_shared_bytes<WT, E>(q.groups, q.n, q.k, b.n_rounds);
-    const RoundScratch scratch = round_scratch(h);
     auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR>;
     if (smem > 48 * 1024)  // more than 16 selected devices
       HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -390,7 +389,7 @@ bool resident_form(const hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b) {
   return 2 * sum_steps <= 3 * (int64_t)n * b.n_rounds ? b.n_rounds >= 4 : n <= 24 && b.n_rounds >= 6;
 }
 
-int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b, float lr) {
+int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b, float lr, const RoundScratch &scratch) {
   return for_storage(h, [&](auto wt, auto mt, auto rm) {
     using WT = typename decltype(wt)::type;
     using MT = typename decltype(mt)::type;
@@ -452,7 +451,6 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
     if (smem < floor_bytes && blocks_per_sm < kResidentMaxBlocks) smem = floor_bytes;
     const int64_t chunks = (h->cfg.n_params + 8 * kResidentThreads - 1) / (8 * kResidentThreads);
     const int grid = (int)(chunks < kRoundGridCap ? chunks : kRoundGridCap);
-    const RoundScratch scratch = round_scratch(h);
     auto kernel = q.n_on_chip == n ? k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, true>
                                    : k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, false>;
     HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -464,17 +462,13 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
 }
 
 template <int NR>
-int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
-  if (rows_form(h, b.n_rounds)) return launch_round_rows<NR>(h, b, lr);
-  if constexpr (NR > 1)
-    if (resident_form(h, b)) return launch_rounds_resident(h, b, lr);
+int launch_round_walk(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const RoundScratch &scratch) {
   return for_storage(h, [&](auto wt, auto mt, auto rm) {
     using WT = typename decltype(wt)::type;
     using MT = typename decltype(mt)::type;
     const size_t smem = sizeof(float) * kThreads * (size_t)h->cfg.n_devices;
     constexpr int E = StepPack<WT>::E;
     constexpr int RM = decltype(rm)::value;
-    const RoundScratch scratch = round_scratch(h);
     int max_steps = 0;
     int64_t sum_steps = 0, n_rows = 0;
     for (int r = 0; r < b.n_rounds; ++r)
@@ -512,6 +506,24 @@ int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
   });
 }
 
+template <int NR>
+int launch_round_form(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const RoundScratch &scratch) {
+  if (rows_form(h, b.n_rounds)) return launch_round_rows<NR>(h, b, lr, scratch);
+  if constexpr (NR > 1)
+    if (resident_form(h, b)) return launch_rounds_resident(h, b, lr, scratch);
+  return launch_round_walk<NR>(h, b, lr, scratch);
+}
+
+template <int NR>
+int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
+  const RoundScratch scratch = round_scratch(h);
+  const int rc = launch_round_form<NR>(h, b, lr, scratch);
+  if (rc != HADFL_OK) return rc;
+  stats_enqueued(h, scratch.out);
+  h->round_stats_at = scratch.out_rounds;
+  return HADFL_OK;
+}
+
 template <typename WT, int KR, int U>
 int launch_combine_as(hadfl_handle *h, const CombineArgs &c) {
   constexpr int E = Pack16<WT>::E;
@@ -537,10 +549,13 @@ int launch_combine(hadfl_handle *h, const CombineArgs &c) {
 
 template <typename WT>
 int launch_stats(hadfl_handle *h, int ref) {
+  float *out = next_stats(h);
   k_stats<WT, kStatsU><<<h->stats_lanes * h->cfg.n_devices, kThreads, 0, h->stream>>>(
       (const WT *)h->w, h->stride, h->cfg.n_params, h->cfg.n_devices, ref, h->stats_lanes,
-      h->d_partials, h->d_ticket, next_stats(h));
-  return check_launch(h);
+      h->d_partials, h->d_ticket, out);
+  const int rc = check_launch(h);
+  if (rc == HADFL_OK) stats_enqueued(h, out);
+  return rc;
 }
 
 int read_row(hadfl_handle *h, int32_t id, float *dst, int64_t count, bool momentum) {
