@@ -954,6 +954,16 @@ __device__ __forceinline__ void finish_two_level(const double *__restrict__ part
   if (threadIdx.x == 0) *ticket = 0u;
 }
 
+// Where statistics go: device memory, and the same place of a buffer in host memory where there is one.  (1 to 2 us
+// at the end of a launch for stores to the host; those to the device beside them cost nothing that shows.)
+struct StatsOut {
+  float *dev, *host;
+  __device__ __forceinline__ void put(int at, float x) const {
+    if (access_ok(dev + at, 4)) dev[at] = x;
+    if (host && access_ok(host + at, 4)) host[at] = x;
+  }
+};
+
 // ------------------------------------------------------------------------------------------
 // K3: per-replica squared norm and squared distance to a reference replica.
 // Block b works on row b % N and on the chunks (b / N), (b / N) + lanes, ...; a chunk is
@@ -969,7 +979,7 @@ template <typename WT, int U>
 __global__ void __launch_bounds__(kThreads)
 k_stats(const WT *__restrict__ w, int64_t stride, int64_t n_params, int n_devices, int ref,
         int lanes, double *__restrict__ partials, unsigned int *__restrict__ ticket,
-        float *__restrict__ out) {
+        StatsOut out) {
   constexpr int kWarps = kThreads / 32;
   constexpr int E = Pack16<WT>::E;
   __shared__ double s_part[2][kWarps];
@@ -1037,9 +1047,7 @@ k_stats(const WT *__restrict__ w, int64_t stride, int64_t n_params, int n_device
     if (access_ok(slot, 8)) *slot = s;
   }
   finish_by_last_block(partials, 2 * n_devices, lanes, ticket, &s_last,
-                       [&](int t, double sum) {
-                         if (access_ok(out + t, 4)) out[t] = (float)sum;
-                       });
+                       [&](int t, double sum) { out.put(t, (float)sum); });
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1123,8 +1131,12 @@ struct RoundScratch {
   double *partials;            // [round][2 n][blocks]
   double *group_partials;      // [round][2 n][groups]
   unsigned int *tickets;       // [1 + groups]: the launch's ticket, then one per group of blocks
-  float *out_rounds;           // [round][2 kMaxDevices]: the statistics of every round of the batch
-  float *out;                  // [2 kMaxDevices]: the statistics of the batch's last round
+  StatsOut out;                // [2 kMaxDevices] of the batch's last round, then as many of each round
+  // value `at` of round r of n_rounds
+  __device__ __forceinline__ void put(int r, int n_rounds, int at, float x) const {
+    out.put((1 + r) * 2 * kMaxDevices + at, x);
+    if (r + 1 == n_rounds) out.put(at, x);
+  }
 };
 
 template <typename WT, typename MT, typename Gen, int E, int RM, bool PF, int NR>
@@ -1293,11 +1305,7 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
                    [&](int t, double sum) {
     const int r = NR == 1 ? 0 : t / (2 * n_dev), v = t - r * 2 * n_dev, j = v >> 1, which = v & 1;
     const RoundArgs &a = b.round[r];
-    float *out_r = scratch.out_rounds + r * 2 * kMaxDevices;
-    auto put = [&](int at, float x) {  // every round's statistics; the last round's also where hadfl_stats puts them
-      if (access_ok(out_r + at, 4)) out_r[at] = x;
-      if (r + 1 == n_rounds && access_ok(scratch.out + at, 4)) scratch.out[at] = x;
-    };
+    auto put = [&](int at, float x) { scratch.put(r, n_rounds, at, x); };
     if (j == a.k - 1) {  // the selected devices share one norm and are at distance 0
       for (int q = 0; q < a.k; ++q) put(which * n_dev + a.r[q].row, which ? 0.f : (float)sum);
     } else if (j >= a.k) {
@@ -1503,9 +1511,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
   finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
                    [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, at = (v & 1) * n + (v >> 1);  // [norms of the rows][distances]
-    float *out_r = scratch.out_rounds + r * 2 * kMaxDevices;
-    if (access_ok(out_r + at, 4)) out_r[at] = (float)sum;
-    if (r + 1 == n_rounds && access_ok(scratch.out + at, 4)) scratch.out[at] = (float)sum;
+    scratch.put(r, n_rounds, at, (float)sum);
   });
 }
 
@@ -1897,11 +1903,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
   finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
                    [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, j = v >> 1, which = v & 1;
-    float *out_r = scratch.out_rounds + r * 2 * kMaxDevices;
-    auto put = [&](int at, float x) {
-      if (access_ok(out_r + at, 4)) out_r[at] = x;
-      if (r + 1 == b.n_rounds && access_ok(scratch.out + at, 4)) scratch.out[at] = x;
-    };
+    auto put = [&](int at, float x) { scratch.put(r, b.n_rounds, at, x); };
     if (j == n_sel - 1) {  // the holders of the aggregate share one norm and are at distance 0
       for (int q = 0; q < (b.write_all[r] == 1 ? n : n_sel); ++q) put(which * n + b.draw[r][q], which ? 0.f : (float)sum);
     } else if (j >= n_sel && b.write_all[r] != 1) {

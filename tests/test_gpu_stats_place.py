@@ -1,5 +1,5 @@
 """Statistics that are read now and then: whether the last launches wrote them to the host or to the device, a
-read returns those of the round it names, also after a launch that failed."""
+read returns those of the round it names - also after a launch that failed, and after a replayed graph."""
 import ctypes
 import glob
 import os
@@ -79,5 +79,35 @@ def test_statistics_stay_readable_after_a_launch_that_failed(call, launches_sinc
         got, want = a.h.stats_read_round(back), same.h.stats_read_round(back)
         assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     assert all(np.array_equal(x, y) for x, y in zip(a.h.get_versions(), same.h.get_versions()))
+    a.close()
+    same.close()
+
+
+@pytest.mark.parametrize("watched", [False, True])    # whether statistics are being read when the graph is captured
+@pytest.mark.parametrize("watched_at_replay", [False, True])
+def test_statistics_of_a_replayed_graph(watched, watched_at_replay):
+    require_gpu()
+    stream = torch.cuda.Stream()
+    wl = Workload("graph", 4, 20_003, 2, 40, "fixed", (1, 2, 3, 4), grad_std=1e-2, seed=workloads.BASE_SEED + 11)
+    a, same = runtime.Arena(wl, stream=stream), runtime.Arena(wl)
+    for r in range(6):
+        a.run_round_fused(r), same.run_round_fused(r)
+    if watched:
+        a.h.stats_read()
+    a.h.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        a.h.stats_enqueue(1)
+    for r in range(6, 18):
+        a.run_round_fused(r), same.run_round_fused(r)
+        if watched_at_replay:
+            a.h.stats_read()
+    graph.replay()
+    torch.cuda.synchronize()
+    same.h.stats_enqueue(1)
+    got, want = a.h.stats_read(), same.h.stats_read()
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    a.h.synchronize()
+    del graph
     a.close()
     same.close()
