@@ -1511,7 +1511,8 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
   finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
                    [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, at = (v & 1) * n + (v >> 1);  // [norms of the rows][distances]
-    scratch.put(r, n_rounds, at, (float)sum);
+    const bool holder = b.s[r][v >> 1].visit < n_sel;  // of the aggregate: at distance 0, whatever its values
+    scratch.put(r, n_rounds, at, holder && (v & 1) ? 0.f : (float)sum);
   });
 }
 
@@ -1822,6 +1823,14 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
           n2 = fmaf(acc[i], acc[i], n2);
         }
         const int write_all = b.write_all[r], n_holders = write_all == 1 ? n : n_sel;
+        float d2_held = 0.f;  // of the devices that are overwritten: as between any two models, NaN where acc is not finite
+        if (write_all == 1) {
+#pragma unroll
+          for (int i = 0; i < E; ++i) {
+            const float d = acc[i] - acc[i];
+            d2_held = fmaf(d, d, d2_held);
+          }
+        }
         {
           RawPack<WT, E> ra;
           pack_raw(acc, ra);
@@ -1829,7 +1838,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
           for (int t = 0; t < n_holders; ++t)
             at_place(b.draw[r][t], [&](auto where, int row) { store_w(where, row, ra); });
         }
-        Sums::add(slots, 0, n2, 0.f, lane);  // one value for all holders
+        Sums::add(slots, 0, n2, d2_held, lane);  // one value for all holders
         // ---- the other devices: keep their own model, or mix the aggregate into it
         int slot = 0;
 #pragma unroll 1
@@ -1904,8 +1913,9 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
                    [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, j = v >> 1, which = v & 1;
     auto put = [&](int at, float x) { scratch.put(r, b.n_rounds, at, x); };
-    if (j == n_sel - 1) {  // the holders of the aggregate share one norm and are at distance 0
-      for (int q = 0; q < (b.write_all[r] == 1 ? n : n_sel); ++q) put(which * n + b.draw[r][q], which ? 0.f : (float)sum);
+    if (j == n_sel - 1) {  // the holders of the aggregate share one norm; the selected ones are at distance 0
+      for (int q = 0; q < (b.write_all[r] == 1 ? n : n_sel); ++q)
+        put(which * n + b.draw[r][q], which && q < n_sel ? 0.f : (float)sum);
     } else if (j >= n_sel && b.write_all[r] != 1) {
       put(which * n + b.draw[r][j], (float)sum);
     }
