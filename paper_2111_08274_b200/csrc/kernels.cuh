@@ -1467,11 +1467,11 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
         }
 #pragma unroll
         for (int i = 0; i < E; ++i) acc[i] = as_stored(acc[i], w);
-        if (j < n_sel || write_all == 1) {
+        if (j < n_sel ? n_sel > 1 || rs.steps > 0 : write_all == 1) {  // (see k_round for the single device without steps)
 #pragma unroll
           for (int i = 0; i < E; ++i) wv[i] = acc[i];
           w_changed = true;
-        } else if (write_all == 2) {
+        } else if (j >= n_sel && write_all == 2) {
 #pragma unroll
           for (int i = 0; i < E; ++i)
             wv[i] = as_stored(fmaf(b.beta, acc[i], __fmul_rn(b.one_minus_beta, wv[i])), w);
@@ -1540,6 +1540,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 // The first step's noise is drawn while the row's values are on their way (434 -> 421 us with everything on
 // the SM, 16 devices).  Each row is either wholly on the SM or wholly in the arena and the code is compiled
 // for either place: choosing at every access cost 100 instructions per row and pack in register copies.
+// Values move between the arena and the SM as they are: NaNs of rows that nothing changes keep their bits.
 // ------------------------------------------------------------------------------------------
 constexpr int kResidentThreads = 128;
 constexpr int kResidentMaxBlocks = 6;  // per SM, by registers (80 a thread); shared memory sets the actual number
@@ -1695,7 +1696,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
         else
           st_raw(at_row<WT>(wp, b.w_off[row]), live, r);
       };
-      auto load_m = [&](auto where, int row, RawPack<MT, E> &r) {  // the values: through m_values
+      auto load_m = [&](auto where, int row, RawPack<MT, E> &r) {  // there after m_arrived
         if constexpr (decltype(where)::value) {
           uint32_t v[kWords];
           tmem_load(tm + row * kWords, v);
@@ -1704,7 +1705,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
           ld_raw(at_row<MT>(mp, b.m_off[row]), live, r);
         }
       };
-      auto m_values = [&](auto where, RawPack<MT, E> &r, float (&mv)[E]) {
+      auto m_arrived = [&](auto where, RawPack<MT, E> &r) {
         if constexpr (decltype(where)::value) {
           uint32_t v[kWords];
           tmem_wait_load();
@@ -1712,11 +1713,8 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
           tmem_use(v);
           memcpy(&r, v, sizeof(v));
         }
-        unpack(r, mv);
       };
-      auto store_m = [&](auto where, int row, const float (&mv)[E]) {
-        RawPack<MT, E> r;
-        pack_raw(mv, r);
+      auto store_m = [&](auto where, int row, const RawPack<MT, E> &r) {
         if constexpr (decltype(where)::value) {
           uint32_t v[kWords];
           memcpy(v, &r, sizeof(v));
@@ -1748,12 +1746,10 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
       for (int row = 0; row < n_on_chip; ++row) {
         RawPack<WT, E> rw;
         RawPack<MT, E> rm;
-        float mv[E];
         ld_raw(at_row<WT>(wp, b.w_off[row]), live, rw);
         load_m(std::false_type{}, row, rm);
-        m_values(std::false_type{}, rm, mv);
         store_w(std::true_type{}, row, rw);
-        store_m(std::true_type{}, row, mv);
+        store_m(std::true_type{}, row, rm);
       }
       tmem_wait_store();
 
@@ -1784,7 +1780,8 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
             // the values are on their way while the first step's noise is drawn
             float2 nz[E / 4][2];
             step_noise<Gen, E / 4>(nz, 0, c2_first, gp, rs, keys, k);
-            m_values(where, rm, mv);
+            m_arrived(where, rm);
+            unpack(rm, mv);
             unpack(rw, wv);
             step_update<E / 4>(wv, mv, nz, k);
 #pragma unroll 1
@@ -1795,7 +1792,8 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
             if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, rs, keys);
             pack_raw(wv, rw);
             store_w(where, row, rw);
-            store_m(where, row, mv);
+            pack_raw(mv, rm);
+            store_m(where, row, rm);
           });
         }
         // ---- aggregation with write-back: acc = a_0 w_0, then acc = fma(a_j, w_j, acc) in draw order
@@ -1834,8 +1832,10 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
         {
           RawPack<WT, E> ra;
           pack_raw(acc, ra);
+          // a single selected device that ran no steps already holds the aggregate (a_0 = 1)
+          const int first = n_sel == 1 && b.s[r][b.draw[r][0]].steps == 0;
 #pragma unroll 1
-          for (int t = 0; t < n_holders; ++t)
+          for (int t = first; t < n_holders; ++t)
             at_place(b.draw[r][t], [&](auto where, int row) { store_w(where, row, ra); });
         }
         Sums::add(slots, 0, n2, d2_held, lane);  // one value for all holders
@@ -1877,12 +1877,11 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
       for (int row = 0; row < n_on_chip; ++row) {
         RawPack<WT, E> rw;
         RawPack<MT, E> rm;
-        float mv[E];
         load_m(std::true_type{}, row, rm);
         load_w(std::true_type{}, row, rw);
-        m_values(std::true_type{}, rm, mv);
+        m_arrived(std::true_type{}, rm);
         st_raw(at_row<WT>(wp, b.w_off[row]), live, rw);
-        store_m(std::false_type{}, row, mv);
+        store_m(std::false_type{}, row, rm);
       }
     };
     if ((chunk + 1) * kResidentThreads * E <= n_params && rows_at_32(w, m))

@@ -53,3 +53,28 @@ def test_statistics(form, sync_every, bad, storage):
         assert np.isfinite(n2[2:]).all() != bool(sync_every)
     a.h.debug_check()
     a.close()
+
+
+@pytest.mark.parametrize("storage", [(0, 0), (1, 0), (1, 1)])
+@pytest.mark.parametrize("form", sorted(FORMS))
+def test_untouched_values_keep_their_bits(form, storage):
+    """NaNs with a payload, and signalling ones, in the parameters and the momentum of devices that run no steps
+    and receive nothing: of the unselected ones, and of the selected one where it is the only one."""
+    n, P, rounds = FORMS[form]
+    wl = Workload("bits", n, P, 1, 1, "fixed", (0,) * n, dtype=storage[0], m_dtype=storage[1],
+                  seed=workloads.BASE_SEED + P)
+    a = runtime.Arena(wl)
+    bits = {4: [0x7FC12345, -0x003EDCBB, 0x7F812345, -0x80000000, 1], 2: [0x7FC5, -0x0035, 0x7F85, -0x8000, 1]}
+    whole = []
+    for t in (a.w, a.m):
+        t = t.view(torch.int32 if t.element_size() == 4 else torch.int16)
+        t[:, :5] = torch.tensor(bits[t.element_size()], dtype=t.dtype, device="cuda")
+        t[:, P - 1] = t[:, 0]
+        whole.append((t, t.clone()))
+    torch.cuda.synchronize()
+    a.run_rounds_fused(0, rounds)
+    torch.cuda.synchronize()
+    for now, before in whole:
+        assert torch.equal(now, before)
+    a.h.debug_check()
+    a.close()
