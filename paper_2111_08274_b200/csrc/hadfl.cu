@@ -30,6 +30,8 @@ struct hadfl_handle {
   int sm_count = 0;
   int l2_bytes = 0;
   size_t smem_per_sm = 0;
+  int smem_per_block = 0;                   // most shared memory of a block, static and dynamic
+  bool rows_smem[2] = {};                   // allow_all_shared is done for k_round_rows (launches of one round, batches)
   size_t resident_arena_bytes = 0;  // batches on arenas beyond this are resident on the SMs
   PhiloxKeys keys;
   uint32_t version[kMaxDevices];
@@ -332,6 +334,21 @@ bool rows_form(const hadfl_handle *h, int n_rounds) {
   return n_rounds > 1 ? work <= ((int64_t)1 << 22) : P <= ((int64_t)1 << 17) && work <= ((int64_t)1 << 21);
 }
 
+// Lets launches of the kernel take all the shared memory that a block can have; which blocks share an SM follows
+// from what a launch asks for.  The limit belongs to the kernel, not to the handle: it is always the same one, so
+// that handles in other threads never find a lower one than they need.  (Without this call a launch gets 48 KB,
+// the kernel's own variables included.)
+template <typename Kernel>
+int allow_all_shared(hadfl_handle *h, Kernel kernel, bool &done) {
+  if (done) return HADFL_OK;
+  cudaFuncAttributes attr;
+  HADFL_CUDA(h, cudaFuncGetAttributes(&attr, kernel));
+  HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     h->smem_per_block - (int)attr.sharedSizeBytes));
+  done = true;
+  return HADFL_OK;
+}
+
 // Rows form: tiles of a block (at least 8 warps) and blocks of a launch.
 int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
 int64_t rows_grid(int n_devices, int64_t n_params) {
@@ -363,8 +380,8 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
     const int grid = (int)rows_grid(q.n, h->cfg.n_params);
     const size_t smem = rows_shared_bytes<WT, E>(q.groups, q.n, q.k, b.n_rounds);
     auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR>;
-    if (smem > 48 * 1024)  // more than 16 selected devices
-      HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int rc = allow_all_shared(h, kernel, h->rows_smem[NR > 1]);
+    if (rc != HADFL_OK) return rc;
     kernel<<<grid, q.groups * q.n * 32, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->stride, h->cfg.n_params, h->keys,
                                                            step_consts(h, lr), scratch, q);
     h->last_launch_pack = E;
@@ -705,6 +722,7 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
     int smem_per_sm = 0;
     HADFL_CUDA(h, cudaDeviceGetAttribute(&smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, h->device));
     h->smem_per_sm = (size_t)smem_per_sm;
+    HADFL_CUDA(h, cudaDeviceGetAttribute(&h->smem_per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     h->resident_arena_bytes = (size_t)h->l2_bytes / 8 * 9;
     const double resident_rows = 4.0 * h->sm_count * cfg->n_devices * (kThreads * 4.0) * 8.0;
     h->round_half_packs = cfg->dtype == HADFL_DTYPE_FP32 && resident_rows <= 0.8 * h->l2_bytes &&
