@@ -32,6 +32,7 @@ struct hadfl_handle {
   size_t smem_per_sm = 0;
   int smem_per_block = 0;                   // most shared memory of a block, static and dynamic
   bool rows_smem[2] = {};                   // allow_all_shared is done for k_round_rows (launches of one round, batches)
+  bool resident_smem[2] = {};               // ... for k_rounds_resident (a part of the rows on the SM, all of them)
   size_t resident_arena_bytes = 0;  // batches on arenas beyond this are resident on the SMs
   PhiloxKeys keys;
   uint32_t version[kMaxDevices];
@@ -475,7 +476,8 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
     const int grid = (int)(chunks < kRoundGridCap ? chunks : kRoundGridCap);
     auto kernel = q.n_on_chip == n ? k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, true>
                                    : k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, false>;
-    HADFL_CUDA(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int rc = allow_all_shared(h, kernel, h->resident_smem[q.n_on_chip == n]);
+    if (rc != HADFL_OK) return rc;
     kernel<<<grid, kResidentThreads, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->cfg.n_params, h->keys,
                                                         step_consts(h, lr), scratch, q);
     h->last_launch_pack = 8;
