@@ -42,16 +42,18 @@ struct hadfl_handle {
   double *d_partials = nullptr;
   unsigned int *d_ticket = nullptr;
   // Statistics: 2 * kMaxDevices floats of the last round, then as many of each round of a batch; one such buffer
-  // in device memory and one in page-locked host memory.  Every launch writes to the device.  While statistics
-  // are being read - within the last kStatsWatch launches that made any - launches write to the host as well
-  // (reading is then a wait for the stream and no copy: a watched round of 4 devices and 100,000 parameters
-  // 43.5 -> 31 us); else not, as stores to the host make the end of a launch 1 to 2 us later (6 devices, 150,001
-  // parameters: 10.6 against 12.4 us).  Launches that a graph captures write to both, so that a replay leaves
-  // the host's copy as right, or as out of date, as it was.
+  // in device memory and one in page-locked host memory.  While statistics are being read - within the last
+  // kStatsWatch launches that made any - launches write to the host (reading is then a wait for the stream and
+  // no copy: a watched round of 4 devices and 100,000 parameters 43.5 -> 31 us), else to the device: stores
+  // to the host make the end of a launch 1 to 2 us later (6 devices, 150,001 parameters: 10.6 against 12.4 us).
+  // From the first launch on that a graph captures, all write where the last one before it did: a replay's
+  // statistics are then found where those before it were.  (Writing to both places instead made ten rounds of 4
+  // devices 65.0 -> 65.9 us, eight of 16 devices and 2^22 bf16 parameters 843 -> 848.)
   float *stats_dev = nullptr, *stats_host = nullptr;
-  bool host_has_last = false;      // the host has the statistics of the last launch with statistics, its (last) round ...
-  bool host_has_rounds = false;    // ... and those of each round of the last launch of the fused round kernel
-  int stats_unread = kStatsWatch;  // launches with statistics since the last read
+  float *stats_at = nullptr;        // where the last launch with statistics wrote those of its (last) round
+  float *round_stats_at = nullptr;  // ... and the last launch of the fused round kernel those of each round
+  bool stats_pinned = false;        // both stay where they are
+  int stats_unread = kStatsWatch;   // launches with statistics since the last read
   int stats_lanes = 0;  // blocks per row of the statistics kernel
   bool stats_valid = false;
   // fused round kernel scratch
@@ -231,25 +233,34 @@ bool capturing(const hadfl_handle *h) {
 
 // Where the next launch writes its statistics, and the note that it has been enqueued (a launch that failed leaves
 // the statistics of the one before it readable).
-StatsOut next_stats(const hadfl_handle *h) {
-  return StatsOut{h->stats_dev, h->stats_unread < kStatsWatch || capturing(h) ? h->stats_host : nullptr};
+struct StatsPlace {
+  float *last, *rounds;
+};
+StatsPlace next_stats(hadfl_handle *h) {
+  if (!h->stats_pinned && capturing(h)) h->stats_pinned = true;
+  if (h->stats_pinned) return StatsPlace{h->stats_at, h->round_stats_at};
+  float *at = h->stats_unread < kStatsWatch ? h->stats_host : h->stats_dev;
+  return StatsPlace{at, at + kStatsFloats};
 }
-void stats_enqueued(hadfl_handle *h, const StatsOut &out, bool rounds) {
-  if (capturing(h)) return;
-  h->host_has_last = out.host != nullptr;
-  if (rounds) h->host_has_rounds = out.host != nullptr;
+void stats_enqueued(hadfl_handle *h, float *last) {
+  h->stats_at = last;
   if (h->stats_unread < kStatsWatch) ++h->stats_unread;
 }
 
-// Waits for the stream and returns the statistics at `at` of the buffers in host memory.
-int fetch_stats(hadfl_handle *h, size_t at, bool on_host, const float **out) {
-  if (!on_host)
-    HADFL_CUDA(h, cudaMemcpyAsync(h->stats_host + at, h->stats_dev + at, sizeof(float) * 2 * (size_t)h->cfg.n_devices,
-                                  cudaMemcpyDeviceToHost, h->stream));
+// Waits for the stream and returns statistics at `at` in host memory.
+int fetch_stats(hadfl_handle *h, const float *at, const float **out) {
+  const float *host = h->stats_host;
+  const bool on_device = at < host || at >= host + kStatsFloats * (1 + kRoundBatchMax);
+  if (on_device) {
+    float *copy = h->stats_host + (at - h->stats_dev);
+    HADFL_CUDA(h, cudaMemcpyAsync(copy, at, sizeof(float) * 2 * (size_t)h->cfg.n_devices, cudaMemcpyDeviceToHost,
+                                  h->stream));
+    at = copy;
+  }
   HADFL_CUDA(h, cudaStreamSynchronize(h->stream));
   HADFL_DEBUG_RESULT();
   h->stats_unread = 0;
-  *out = h->stats_host + at;
+  *out = at;
   return HADFL_OK;
 }
 
@@ -540,10 +551,13 @@ int launch_round_form(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
 
 template <int NR>
 int launch_round(hadfl_handle *h, const RoundBatch<NR> &b, float lr) {
-  const RoundScratch scratch{h->d_round_partials, h->d_round_group_partials, h->d_round_ticket, next_stats(h)};
-  const int rc = launch_round_form<NR>(h, b, lr, scratch);
-  if (rc == HADFL_OK) stats_enqueued(h, scratch.out, true);
-  return rc;
+  const StatsPlace to = next_stats(h);
+  const int rc = launch_round_form<NR>(h, b, lr, RoundScratch{h->d_round_partials, h->d_round_group_partials,
+                                                              h->d_round_ticket, to.rounds, to.last});
+  if (rc != HADFL_OK) return rc;
+  stats_enqueued(h, to.last);
+  h->round_stats_at = to.rounds;
+  return HADFL_OK;
 }
 
 template <typename WT, int KR, int U>
@@ -571,12 +585,12 @@ int launch_combine(hadfl_handle *h, const CombineArgs &c) {
 
 template <typename WT>
 int launch_stats(hadfl_handle *h, int ref) {
-  const StatsOut out = next_stats(h);
+  float *out = next_stats(h).last;
   k_stats<WT, kStatsU><<<h->stats_lanes * h->cfg.n_devices, kThreads, 0, h->stream>>>(
       (const WT *)h->w, h->stride, h->cfg.n_params, h->cfg.n_devices, ref, h->stats_lanes,
       h->d_partials, h->d_ticket, out);
   const int rc = check_launch(h);
-  if (rc == HADFL_OK) stats_enqueued(h, out, false);
+  if (rc == HADFL_OK) stats_enqueued(h, out);
   return rc;
 }
 
@@ -703,6 +717,8 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
   HADFL_CUDA(h, cudaMemsetAsync(h->stats_dev, 0, stats_bytes, h->stream));
   HADFL_CUDA(h, cudaHostAlloc((void **)&h->stats_host, stats_bytes, cudaHostAllocMapped));
   memset(h->stats_host, 0, stats_bytes);
+  h->stats_at = h->stats_dev;
+  h->round_stats_at = h->stats_dev + kStatsFloats;
   // Fused round kernel: one block per chunk of kThreads packs (8 columns each) up to kRoundGridCap
   // blocks, beyond which the blocks stride over the chunks.  Measured on the workloads' sizes, a grid
   // of many short blocks beats one resident wave by 7-15 % with several steps per device and is
@@ -1181,7 +1197,7 @@ int hadfl_stats_read_round(hadfl_handle *h, int32_t back, float *out_norm2, floa
   DeviceGuard guard(h->device);
   const int n = h->cfg.n_devices;
   const float *src = nullptr;
-  const int rc = fetch_stats(h, (size_t)(h->last_launch_rounds - back) * kStatsFloats, h->host_has_rounds, &src);
+  const int rc = fetch_stats(h, h->round_stats_at + (size_t)(h->last_launch_rounds - 1 - back) * kStatsFloats, &src);
   if (rc != HADFL_OK) return rc;
   memcpy(out_norm2, src, sizeof(float) * (size_t)n);
   memcpy(out_div2, src + n, sizeof(float) * (size_t)n);
@@ -1203,7 +1219,7 @@ int hadfl_stats_read(hadfl_handle *h, float *out_norm2, float *out_div2) {
   DeviceGuard guard(h->device);
   const int n = h->cfg.n_devices;
   const float *src = nullptr;
-  const int rc = fetch_stats(h, 0, h->host_has_last, &src);
+  const int rc = fetch_stats(h, h->stats_at, &src);
   if (rc != HADFL_OK) return rc;
   memcpy(out_norm2, src, sizeof(float) * (size_t)n);
   memcpy(out_div2, src + n, sizeof(float) * (size_t)n);
@@ -1295,11 +1311,11 @@ int hadfl_stats_noalloc(const void *w, int32_t dtype, int32_t n_devices, int64_t
   if (dtype == HADFL_DTYPE_BF16)
     k_stats<__nv_bfloat16, kStatsU><<<blocks, kThreads, 0, stream>>>(
         (const __nv_bfloat16 *)w, row_stride_elems, n_params, n_devices, ref_device, (int)lanes,
-        partials, ticket, StatsOut{out_stats, nullptr});
+        partials, ticket, out_stats);
   else
     k_stats<float, kStatsU><<<blocks, kThreads, 0, stream>>>(
         (const float *)w, row_stride_elems, n_params, n_devices, ref_device, (int)lanes, partials,
-        ticket, StatsOut{out_stats, nullptr});
+        ticket, out_stats);
   return cudaGetLastError() == cudaSuccess ? HADFL_OK : HADFL_ERR_CUDA;
 }
 

@@ -954,16 +954,6 @@ __device__ __forceinline__ void finish_two_level(const double *__restrict__ part
   if (threadIdx.x == 0) *ticket = 0u;
 }
 
-// Where statistics go: device memory, and the same place of a buffer in host memory where there is one.  (1 to 2 us
-// at the end of a launch for stores to the host; those to the device beside them cost nothing that shows.)
-struct StatsOut {
-  float *dev, *host;
-  __device__ __forceinline__ void put(int at, float x) const {
-    if (access_ok(dev + at, 4)) dev[at] = x;
-    if (host && access_ok(host + at, 4)) host[at] = x;
-  }
-};
-
 // ------------------------------------------------------------------------------------------
 // K3: per-replica squared norm and squared distance to a reference replica.
 // Block b works on row b % N and on the chunks (b / N), (b / N) + lanes, ...; a chunk is
@@ -979,7 +969,7 @@ template <typename WT, int U>
 __global__ void __launch_bounds__(kThreads)
 k_stats(const WT *__restrict__ w, int64_t stride, int64_t n_params, int n_devices, int ref,
         int lanes, double *__restrict__ partials, unsigned int *__restrict__ ticket,
-        StatsOut out) {
+        float *__restrict__ out) {
   constexpr int kWarps = kThreads / 32;
   constexpr int E = Pack16<WT>::E;
   __shared__ double s_part[2][kWarps];
@@ -1047,7 +1037,9 @@ k_stats(const WT *__restrict__ w, int64_t stride, int64_t n_params, int n_device
     if (access_ok(slot, 8)) *slot = s;
   }
   finish_by_last_block(partials, 2 * n_devices, lanes, ticket, &s_last,
-                       [&](int t, double sum) { out.put(t, (float)sum); });
+                       [&](int t, double sum) {
+                         if (access_ok(out + t, 4)) out[t] = (float)sum;
+                       });
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1131,11 +1123,13 @@ struct RoundScratch {
   double *partials;            // [round][2 n][blocks]
   double *group_partials;      // [round][2 n][groups]
   unsigned int *tickets;       // [1 + groups]: the launch's ticket, then one per group of blocks
-  StatsOut out;                // [2 kMaxDevices] of the batch's last round, then as many of each round
+  float *out_rounds;           // [round][2 kMaxDevices]: the statistics of every round of the batch
+  float *out;                  // [2 kMaxDevices]: the statistics of the batch's last round
   // value `at` of round r of n_rounds
   __device__ __forceinline__ void put(int r, int n_rounds, int at, float x) const {
-    out.put((1 + r) * 2 * kMaxDevices + at, x);
-    if (r + 1 == n_rounds) out.put(at, x);
+    float *out_r = out_rounds + r * 2 * kMaxDevices;
+    if (access_ok(out_r + at, 4)) out_r[at] = x;
+    if (r + 1 == n_rounds && access_ok(out + at, 4)) out[at] = x;
   }
 };
 
