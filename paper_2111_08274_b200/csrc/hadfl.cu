@@ -455,6 +455,7 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
         q.order[r][at] = rs.row;
       }
       q.n_stepping[r] = n_stepping;
+      q.first_store[r] = a.k == 1 && a.r[0].steps == 0;  // it ran no steps, and a_0 = 1
     }
     const int64_t mean_steps_x2 = 2 * sum_steps / ((int64_t)n * b.n_rounds);
     // Blocks per SM.  With more than two steps per device on average the launch is bound by arithmetic, and 6

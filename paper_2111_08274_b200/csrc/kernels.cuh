@@ -1544,6 +1544,7 @@ struct ResidentBatch {
   int32_t n_on_chip;  // devices 0 .. n_on_chip - 1 live on the SM, the others in the arena
   float beta, one_minus_beta;
   int32_t write_all[kRoundBatchMax];                // as in RoundArgs
+  int32_t first_store[kRoundBatchMax];              // 1 where a single selected device holds the aggregate already
   int32_t n_stepping[kRoundBatchMax];               // devices that run at least one step ...
   int32_t order[kRoundBatchMax][kMaxDevices];       // ... by descending step count
   int32_t draw[kRoundBatchMax][kMaxDevices];        // devices: the selected ones in draw order, then the rest
@@ -1815,21 +1816,16 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
           n2 = fmaf(acc[i], acc[i], n2);
         }
         const int write_all = b.write_all[r], n_holders = write_all == 1 ? n : n_sel;
-        float d2_held = 0.f;  // of the devices that are overwritten: as between any two models, NaN where acc is not finite
+        float d2_held = 0.f;  // of the devices that are overwritten: as (acc - acc)^2, NaN where acc is not finite
         if (write_all == 1) {
 #pragma unroll
-          for (int i = 0; i < E; ++i) {
-            const float d = acc[i] - acc[i];
-            d2_held = fmaf(d, d, d2_held);
-          }
+          for (int i = 0; i < E; ++i) d2_held = fmaf(acc[i], 0.f, d2_held);
         }
         {
           RawPack<WT, E> ra;
           pack_raw(acc, ra);
-          // a single selected device that ran no steps already holds the aggregate (a_0 = 1)
-          const int first = n_sel == 1 && b.s[r][b.draw[r][0]].steps == 0;
 #pragma unroll 1
-          for (int t = first; t < n_holders; ++t)
+          for (int t = b.first_store[r]; t < n_holders; ++t)
             at_place(b.draw[r][t], [&](auto where, int row) { store_w(where, row, ra); });
         }
         Sums::add(slots, 0, n2, d2_held, lane);  // one value for all holders
