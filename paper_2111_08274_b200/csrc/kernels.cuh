@@ -1321,7 +1321,7 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
 // On large vectors the waits at the barrier, where all warps of a group are in the same phase, cost more
 // than registers save; there k_round is the faster one (the host decides: see rows_form).
 // A row moves to another warp from block to block, so that the heavy rows meet all SM sub-partitions.
-// Sums of a row: fp32 within the tile (pack in order, then a fixed tree), fp64 beyond.
+// Sums of a row: the fp32 part of the order is k_round's (a thread's pack, then the lanes l and l ^ 16), fp64 beyond.
 // ------------------------------------------------------------------------------------------
 constexpr int kRowsMaxThreads = 1024;
 
@@ -1479,10 +1479,10 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
           d2 = fmaf(d, d, d2);
         }
         const bool upper = (lane & 16) != 0;
-        float v = (upper ? d2 : n2) + __shfl_xor_sync(0xFFFFFFFFu, upper ? n2 : d2, 16);
+        double d = (double)((upper ? d2 : n2) + __shfl_xor_sync(0xFFFFFFFFu, upper ? n2 : d2, 16));
 #pragma unroll
-        for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
-        if ((lane & 15) == 0) sums[r * 2 * n + (lane >> 4)] += (double)v;  // lower half-warp norms, upper distances
+        for (int off = 8; off > 0; off >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, off);
+        if ((lane & 15) == 0) sums[r * 2 * n + (lane >> 4)] += d;  // lower half-warp norms, upper distances
       }
       if (w_changed) st_pack_any(wp, 0, live, wv);
       if (m_changed) st_pack_any(mp, 0, live, mv);
