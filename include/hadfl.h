@@ -338,8 +338,9 @@ uint64_t hadfl_launch_count(const hadfl_handle *h);
 /* Row stride, in elements, of the handle's arenas. */
 int64_t hadfl_row_stride(const hadfl_handle *h);
 
-/* Number of thread blocks one hadfl_round launch of this handle uses (diagnostics; each block works
- * on chunks of 2048 consecutive parameters of every device). */
+/* Number of thread blocks one hadfl_round launch of this handle uses (diagnostics).  Each block works on
+ * chunks of 2048 consecutive parameters of every device; with at most 2^17 parameters and n_devices *
+ * n_params <= 2^21 on tiles of 256, max(8 / n_devices, 1) of them at a time. */
 int32_t hadfl_round_grid(const hadfl_handle *h);
 
 /* ---- host-only functions (no handle, no GPU) ------------------------------------------------- */

@@ -1454,7 +1454,10 @@ int hadfl_debug_range_holds(uint64_t lo, uint64_t hi, uint64_t addr, uint64_t nb
 int hadfl_last_cuda_error(const hadfl_handle *h) { return h ? h->last_cuda_error : 0; }
 uint64_t hadfl_launch_count(const hadfl_handle *h) { return h ? h->launches : 0; }
 int64_t hadfl_row_stride(const hadfl_handle *h) { return h ? h->stride : 0; }
-int32_t hadfl_round_grid(const hadfl_handle *h) { return h ? h->round_grid : 0; }
+int32_t hadfl_round_grid(const hadfl_handle *h) {
+  if (!h) return 0;
+  return rows_form(h, 1) ? (int32_t)rows_grid(h->cfg.n_devices, h->cfg.n_params) : h->round_grid;
+}
 
 int hadfl_selection_probs(const double *x, const uint8_t *avail, int32_t n, double *out_P) {
   if (!x || !out_P || n < 1 || n > HADFL_MAX_DEVICES) return HADFL_ERR_INVALID;

@@ -73,3 +73,12 @@ def test_row_sums_beyond_a_lane_pair_are_in_64_bits(rounds):
         n2, d2 = a.h.stats_read_round(back)
         assert abs(n2[1] - want) <= 2.0 ** -23 * want and abs(d2[1] - want) <= 2.0 ** -23 * want
     a.close()
+
+
+@pytest.mark.parametrize("n,P", [(1, 1), (1, 2049), (3, 1_025), (4, 100_000), (8, 131_072), (32, 65_537), (4, 131_073), (32, 131_072)])
+def test_reported_grid_is_that_of_a_single_round(n, P):
+    a = runtime.Arena(Workload("grid", n, P, 1, 1, "fixed", (1,) * n))
+    rows = P <= 1 << 17 and n * P <= 1 << 21
+    columns = 256 * max(8 // n, 1) if rows else 2048
+    assert a.h.round_grid() == -(-P // columns)
+    a.close()
