@@ -66,8 +66,11 @@ struct hadfl_handle {
   int round_batch = kRoundBatchMax;  // most rounds that hadfl_rounds puts into one launch (1: never batch)
   int last_launch_rounds = 0;        // rounds in the most recent launch of the fused round kernel
   int last_launch_pack = 0;          // columns per thread in that launch
-  // model backup that overlaps with later rounds: staging row (fp32) + copy stream
-  float *d_backup = nullptr;
+  // model backup that overlaps with later rounds: staging row + copy stream
+  void *d_backup = nullptr;
+  size_t backup_elem = 4;        // bytes per staged parameter: 2 where memory is too short to widen bf16 on the device
+  float *backup_dst = nullptr;   // of the backup in flight
+  int64_t backup_count = 0;
   cudaStream_t backup_stream = nullptr;
   cudaEvent_t backup_ready = nullptr, backup_done = nullptr;
   bool backup_in_flight = false;
@@ -1346,6 +1349,15 @@ int hadfl_backup_wait(hadfl_handle *h) {
   DeviceGuard guard(h->device);
   HADFL_CUDA(h, cudaEventSynchronize(h->backup_done));
   h->backup_in_flight = false;
+  if (h->backup_elem == 2) {  // bf16 values in the buffer's upper half: from the front on none is overwritten unread
+    const char *bf16 = (const char *)h->backup_dst + 2 * (size_t)h->backup_count;
+    for (int64_t p = 0; p < h->backup_count; ++p) {
+      uint16_t v;
+      memcpy(&v, bf16 + 2 * p, 2);
+      const uint32_t bits = (uint32_t)v << 16;
+      memcpy(h->backup_dst + p, &bits, 4);
+    }
+  }
   return HADFL_OK;
 }
 
@@ -1359,9 +1371,16 @@ int hadfl_backup_begin(hadfl_handle *h, int32_t device_id, float *dst, int64_t c
   }
   DeviceGuard guard(h->device);
   if (!h->backup_stream) {  // first use: staging row, copy stream, two events
-    HADFL_CUDA(h, cudaMalloc((void **)&h->d_backup, sizeof(float) * (size_t)h->cfg.n_params));
+    cudaError_t e = cudaMalloc(&h->d_backup, h->backup_elem * (size_t)h->cfg.n_params);
+    if (e == cudaErrorMemoryAllocation && h->cfg.dtype == HADFL_DTYPE_BF16) {
+      cudaGetLastError();
+      h->backup_elem = 2;  // as stored: half the memory, but the host widens, in hadfl_backup_wait
+      e = cudaMalloc(&h->d_backup, h->backup_elem * (size_t)h->cfg.n_params);
+      if (e != cudaSuccess) h->backup_elem = 4;
+    }
+    HADFL_CUDA(h, e);
 #ifdef HADFL_DEBUG
-    debug_add(h->d_backup, sizeof(float) * (size_t)h->cfg.n_params);
+    debug_add(h->d_backup, h->backup_elem * (size_t)h->cfg.n_params);
     HADFL_CUDA(h, cudaDeviceSynchronize());
     if (debug_publish()) return HADFL_ERR_CUDA;
 #endif
@@ -1375,21 +1394,24 @@ int hadfl_backup_begin(hadfl_handle *h, int32_t device_id, float *dst, int64_t c
   // backup each, us, widened by the host / here: 9 devices, 33.5 M parameters 76768 / 8256; 28 devices,
   // 758,723: 2356 / 626; 4 devices, 65,537: 236 / 115 for two).
   const int64_t first = (int64_t)device_id * h->stride;
-  if (h->cfg.dtype == HADFL_DTYPE_BF16) {
+  const size_t bytes = h->backup_elem * (size_t)count;
+  if (elem_size(h) < h->backup_elem) {
     const unsigned blocks = (unsigned)((count + 8 * kThreads - 1) / (8 * kThreads));
-    k_widen<<<blocks, kThreads, 0, h->stream>>>((const __nv_bfloat16 *)h->w + first, h->d_backup, count);
+    k_widen<<<blocks, kThreads, 0, h->stream>>>((const __nv_bfloat16 *)h->w + first, (float *)h->d_backup, count);
     const int rc = check_launch(h);
     if (rc != HADFL_OK) return rc;
   } else {
-    HADFL_CUDA(h, cudaMemcpyAsync(h->d_backup, (const float *)h->w + first, sizeof(float) * (size_t)count,
+    HADFL_CUDA(h, cudaMemcpyAsync(h->d_backup, (const char *)h->w + first * (int64_t)elem_size(h), bytes,
                                   cudaMemcpyDeviceToDevice, h->stream));
   }
   HADFL_CUDA(h, cudaEventRecord(h->backup_ready, h->stream));
   HADFL_CUDA(h, cudaStreamWaitEvent(h->backup_stream, h->backup_ready, 0));
-  HADFL_CUDA(h, cudaMemcpyAsync(dst, h->d_backup, sizeof(float) * (size_t)count, cudaMemcpyDeviceToHost,
-                                h->backup_stream));
+  HADFL_CUDA(h, cudaMemcpyAsync((char *)dst + (sizeof(float) * (size_t)count - bytes), h->d_backup, bytes,
+                                cudaMemcpyDeviceToHost, h->backup_stream));
   HADFL_CUDA(h, cudaEventRecord(h->backup_done, h->backup_stream));
   h->backup_in_flight = true;
+  h->backup_dst = dst;
+  h->backup_count = count;
   return HADFL_OK;
 }
 

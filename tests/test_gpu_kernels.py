@@ -426,6 +426,35 @@ def test_backup_widens_bf16_on_the_device(count, m_dtype):
     h.debug_check()
 
 
+def test_backup_of_bf16_where_memory_is_short():
+    """A row of 2^29 bf16 parameters and 1.5 GiB of free device memory: not enough for a staging row of fp32
+    values, enough for one as stored."""
+    P, count = 1 << 29, 100_003
+    wl = Workload("short", 1, P, 1, 1, "fixed", (1,), dtype=1, m_dtype=1, seed=3)
+    h = gpu(wl)
+    values = np.random.default_rng(5).standard_normal(count).astype(np.float32)
+    values[:5] = [0.0, -0.0, np.inf, -np.inf, 1e-39]
+    h.write_params(0, values)
+    want = h.read_params(0, count=count)
+    buf = torch.full((count + 8,), 5.0).pin_memory()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    filler = torch.empty(free - (3 << 29), dtype=torch.uint8, device="cuda")
+    try:
+        assert torch.cuda.mem_get_info()[0] < 4 * P
+        for _ in range(2):
+            h.backup_begin(0, buf, count=count)
+            h.write_params(0, -values)                 # the backup is a snapshot
+            h.backup_wait()
+            assert np.array_equal(buf.numpy()[:count].view(np.uint32), want.view(np.uint32))
+            assert (buf.numpy()[count:] == 5.0).all()
+            h.write_params(0, values)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    h.debug_check()
+
+
 @pytest.mark.parametrize("dtype", [0, 1])
 def test_overlapped_backup_is_a_snapshot(dtype):
     """hadfl_backup_begin captures the row as it is at that point of the stream, even though later
