@@ -7,7 +7,7 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <atomic>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -267,14 +267,32 @@ int fetch_stats(hadfl_handle *h, const float *at, const float **out) {
   return HADFL_OK;
 }
 
-// Page-locks 64 bytes per device once per process, so that the driver's pool of page-locked memory outlives
-// the handles: a handle's statistics then cost 1 us to allocate instead of 1 ms.  Nothing ever uses the bytes;
-// where this fails, handles are only slower to make.
+// 64 page-locked bytes per device that stay from the first handle until the library is unloaded, so that the driver
+// keeps what it has page-locked and a handle's statistics buffer takes 2 us to allocate instead of 2.5 ms.  Nothing
+// uses the bytes; where they are not to be had, or a driver does not behave like that, handles are only slower to make.
+class HostPool {
+ public:
+  void keep(int device) {
+    if (device >= kDevices) return;
+    std::lock_guard<std::mutex> lock(mutex_);
+    if (!block_[device] && cudaHostAlloc(&block_[device], 64, cudaHostAllocMapped) != cudaSuccess) {
+      block_[device] = nullptr;
+      cudaGetLastError();
+    }
+  }
+  ~HostPool() {
+    for (void *b : block_)
+      if (b) cudaFreeHost(b);
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::mutex mutex_;
+  void *block_[kDevices] = {};
+};
 void keep_host_pool(int device) {
-  static std::atomic<uint64_t> kept{0};
-  if (device >= 64 || (kept.fetch_or((uint64_t)1 << device) >> device & 1)) return;
-  void *unused = nullptr;
-  if (cudaHostAlloc(&unused, 64, cudaHostAllocMapped) != cudaSuccess) cudaGetLastError();
+  static HostPool pool;  // made after the runtime has been called, so taken down before the runtime is
+  pool.keep(device);
 }
 
 bool distinct_ids(const hadfl_handle *h, const int32_t *ids, int n) {
