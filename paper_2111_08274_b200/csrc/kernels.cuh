@@ -1886,7 +1886,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
     __syncthreads();
     for (int t = threadIdx.x; t < n_vals; t += kResidentThreads) {  // a value belongs to one thread
       double *at = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
-      double sum = chunk == blockIdx.x ? 0.0 : *at;
+      double sum = chunk == blockIdx.x || !access_ok(at, 8) ? 0.0 : *at;
       if (has_sum(t))
         for (int wi = 0; wi < kWarps; ++wi) sum += lines[wi * n_vals + t];
       if (access_ok(at, 8)) *at = sum;
