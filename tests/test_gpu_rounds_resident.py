@@ -2,8 +2,10 @@
 launched one by one, bit for bit: arenas beyond the L2 with all rows on the SM (few devices), with part of
 them (16 devices and more), light and heavy steps, every storage, ragged ends, odd numbers of rounds,
 global synchronisation by overwriting and by mixing, devices that run no steps, one and all devices
-selected; and small arenas of at most 8 devices, which take the form as well.  The statistics' fp64 sums
-are added in another order: equal to one rounding of the fp32 output."""
+selected; small arenas of at most 8 devices, which take the form as well; and vectors of more chunks than a
+launch has blocks.  The statistics of every round of every launch are compared, those of synchronised rounds
+and of rounds inside a batch among them: their fp64 sums are added in another order, and the output is one
+fp32 rounding of them."""
 import numpy as np
 import pytest
 import torch
@@ -33,19 +35,24 @@ def compare(n, P, k, steps, storage, beta, batches, launches):
     for a in (batch, single):                     # what lies behind the vector must stay as it is
         a.w[:, P:] = 3.0
         a.m[:, P:] = 5.0
-    before, first, got = batch.h.launch_count(), 0, []
+    before, first = batch.h.launch_count(), 0
     for count in batches:
-        got.append(batch.run_rounds_fused(first, count))
+        got = batch.run_rounds_fused(first, count)
+        stats = []
+        for r in range(first, first + count):
+            want = single.run_rounds_fused(r, 1)
+            assert np.array_equal(got[r - first], want[0])
+            stats.append(single.h.stats_read())
+        one_launch = launches == len(batches)
+        for back in range(count if one_launch else 1):
+            a, b = batch.h.stats_read_round(back), stats[count - 1 - back]
+            assert np.allclose(a[0], b[0], rtol=2.0 ** -23, atol=0) and np.allclose(a[1], b[1], rtol=2.0 ** -23, atol=0)
         first += count
     assert batch.h.launch_count() - before == launches
-    want = single.run_rounds_fused(0, rounds)
-    assert np.array_equal(np.concatenate(got), want)
     torch.cuda.synchronize()
     assert torch.equal(batch.w, single.w) and torch.equal(batch.m, single.m)
     va, vb = batch.h.get_versions(), single.h.get_versions()
     assert np.array_equal(va[0], vb[0]) and np.array_equal(va[1], vb[1])
-    a, b = batch.h.stats_read(), single.h.stats_read()
-    assert np.allclose(a[0], b[0], rtol=2.0 ** -23, atol=0) and np.allclose(a[1], b[1], rtol=2.0 ** -23, atol=0)
     batch.h.debug_check()
     batch.close()
     single.close()
@@ -57,12 +64,23 @@ def compare(n, P, k, steps, storage, beta, batches, launches):
 def test_large_arenas(n, k, hi, storage):
     rounding = STORAGE[storage][2]
     P = 150_000_001 // (n * STORAGE[storage][3]) // 1024 * 1024 + {2: 1, 5: 1023, 8: 8, 13: 519}.get(n, 0)
-    steps = tuple((3 * i + 1) % (hi + 1) for i in range(n))
-    compare(n, P, k, steps, storage, 0.25 if n % 2 else 1.0, (8, 3, 1),
-            12 if rounding and n > 16 else 3)   # stochastic rounding with many devices: one by one
+    steps = tuple(i % (hi + 1) for i in range(n))
+    compare(n, P, k, steps, storage, 0.25 if n % 2 else 1.0, (8, 7),
+            15 if rounding and n > 16 else 2)   # stochastic rounding with many devices: one by one
+
+
+@pytest.mark.parametrize("storage", ["fp32", "bf16"])
+def test_two_steps_of_24_devices(storage):
+    compare(24, 150_000_001 // (24 * STORAGE[storage][3]), 5, (2,) * 24, storage, 0.5, (8, 6), 2)
 
 
 @pytest.mark.parametrize("n,P,k", [(8, 524_289, 4), (3, 1_500_007, 2), (1, 4_200_001, 1), (8, 1_048_576, 8)])
 @pytest.mark.parametrize("hi", [1, 6])
 def test_small_arenas(n, P, k, hi):
-    compare(n, P, k, tuple((3 * i + 1) % (hi + 1) for i in range(n)), "fp32", 0.5, (2, 7), 2)
+    compare(n, P, k, tuple(i % (hi + 1) for i in range(n)), "fp32", 0.5, (2, 7), 2)
+
+
+@pytest.mark.parametrize("n,k,beta", [(2, 1, 1.0), (3, 2, 0.25)])
+def test_more_chunks_than_blocks(n, k, beta):
+    """16,384 blocks and chunks of 1024 parameters: each block has a second chunk, a few a third."""
+    compare(n, 2 * 16_384 * 1024 + 5_003, k, tuple(1 + i % 2 for i in range(n)), "bf16_m16", beta, (3,), 1)
