@@ -427,20 +427,46 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
 // devices.  Measured, us per round, row walk / resident (one step, then 1..4 steps per device): 8 devices
 // 1,048,576 parameters 22.3 / 16.3, 29.0 / 26.3; 2.5 M 36.8 / 32.8, 70.8 / 56.4; 16 devices 524,288: 21.9 /
 // 23.4, 32.6 / 35.2; 1,048,576 (the arena is about the L2): 34.7 / 37 and more; 32 devices 262,144: 26.9 / 37.
-// Large arenas of up to 16 devices gain with any number of rounds (1.5e8 parameters in all: 2 rounds 0.98 .. 1.12
-// times the speed, 8 rounds 1.02 .. 1.37).  With more devices half the rows and more stay in L2 while few
-// blocks share an SM, so the form has to save several rounds' traffic: 32 devices, one step, 2 / 3 / 4 /
-// 8 rounds 435 / 436 / 435 / 440 -> 487 / 422 / 383 / 352; two steps 411 .. 415 -> 561 / 511 / 485 / 460; 24
-// devices, two steps, 2 / 4 / 6 / 8 rounds 414 .. 416 -> 472 / 420 / 398 / 396.
+// Large arenas of up to 16 devices gain with any number of rounds at two steps per device or fewer; with more, the
+// way of the rows to the SM and back, under which nothing is computed, has to be spread over several rounds
+// (resident_min_rounds).
+// With more devices half the rows and more stay in L2 while few blocks share an SM, so the form has to save several
+// rounds' traffic: 32 devices, one step, 2 / 3 / 4 / 8 rounds 435 / 436 / 435 / 440 -> 487 / 422 / 383 / 352; two
+// steps 411 .. 415 -> 561 / 511 / 485 / 460; 24 devices, two steps, 2 / 4 / 6 / 8 rounds 414 .. 416 -> 472 / 420 /
+// 398 / 396.
+constexpr int kNever = kRoundBatchMax + 1;
+
+// Rounds that a batch of up to 16 devices needs.  Measured on arenas of 180 MB, 400 MB and 1.2 GB, time of single
+// launches over time of the batch, for 2 / 3 / 4 / 6 / 8 rounds:
+//   fp32, steps 1,1,2,2,4,4,8,8: 8 devices 0.96 / 0.99 / 1.01 / 1.03 / 1.04, 14: 0.93 / 0.97 / 0.98 / 1.00 / 1.00;
+//     1..4: 10 devices 1.03 / 1.09 / 1.12 / 1.13 / 1.14, 14: 0.95 / 1.01 / 0.99 / 1.02 / 1.03;
+//     uniform 1..8: 6 devices 0.99 / 1.01 / 1.04 / 1.05 / 1.06, 10: 0.97 / 1.00 / 1.01 / 1.03 / 1.04, 14: 0.93 / 0.95 /
+//     0.96 / 0.98 / 0.98, 16 (180 MB) 0.90 / 0.94 / 0.96
+//   bf16 parameters, uniform 1..8: 14 devices 1.00 / 1.02 / 1.03 / 1.05 / 1.05, 16: 0.99 / 1.01 / 1.01 / 1.03 / 1.03
+//   bf16 throughout, stochastic rounding: 14 devices, uniform 1..8 0.99 / 1.00 / 1.01 / 1.02 / 1.01; 16, two steps
+//     0.98 / 0.99 / 1.00 / 1.03 / 1.03, uniform 1..8 0.98 / 0.98 / 0.98 / 0.99 / 0.99
+int resident_min_rounds(const hadfl_handle *h, double mean_steps) {
+  const int n = h->cfg.n_devices;
+  if (h->cfg.rounding == HADFL_ROUND_STOCHASTIC) {
+    if (n <= 12 || mean_steps <= 1.5) return 2;
+    return n <= 14 ? 3 : (mean_steps <= 3.0 ? 6 : kNever);
+  }
+  if (mean_steps <= 2.0) return 2;
+  if (h->cfg.dtype == HADFL_DTYPE_BF16) return n <= 14 || mean_steps <= 3.0 ? 2 : 3;
+  if (mean_steps <= 3.0) return n <= 10 ? 2 : 4;
+  if (n <= 6) return 3;
+  return n <= 10 || mean_steps <= 4.0 ? 6 : kNever;
+}
+
 bool resident_form(const hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b) {
   const size_t arena = arena_bytes(h);
   const int n = h->cfg.n_devices;
   if (arena <= kBatchSmallArenaBytes) return n <= 8;
   if (arena <= h->resident_arena_bytes) return false;
-  if (n <= 16) return true;
   int64_t sum_steps = 0;
   for (int r = 0; r < b.n_rounds; ++r)
     for (int j = 0; j < n; ++j) sum_steps += b.round[r].r[j].steps;
+  if (n <= 16) return b.n_rounds >= resident_min_rounds(h, (double)sum_steps / ((double)n * b.n_rounds));
   return 2 * sum_steps <= 3 * (int64_t)n * b.n_rounds ? b.n_rounds >= 4 : n <= 24 && b.n_rounds >= 6;
 }
 
@@ -1086,23 +1112,38 @@ int round_by_separate_calls(hadfl_handle *h, const int32_t *device_ids, const in
   return rc;
 }
 
-// Whether hadfl_rounds may put a planned round into a launch together with its neighbours.
-//   - Arenas of at most 64 MiB, where launches and latency are the cost: always.
-//   - Where batches are resident and at most 16 devices leave most rows on the SM: always (16 devices, 14.7 M,
-//     steps 1,1,2,2,4,4,8,8: 863 -> 822 us per round, bf16 parameters 859 -> 816; 8 devices, 11.2 M, 1..8 steps
-//     360 -> 345; but 32 devices, 12 M, 1..4 steps 1165 -> 1269).
-//   - Else rounds of at most two steps per device, which are bound by memory, and only with rounding to nearest
-//     even: stochastic rounding draws a second random block per pack and call (row walk -3 ... -5 %; resident
-//     with 24 and 32 devices -6 ... +2 %).  With more steps the row walk gains nothing (0 ... -3 %).
-bool batchable(const hadfl_handle *h, const RoundPlan &pl) {
+// Rounds that hadfl_rounds puts into one launch:
+//   - On arenas of at most 64 MiB, where launches and latency are the cost: all.
+//   - On arenas of at most 16 devices whose batches are resident: all, where the batch is one that gains from it
+//     (resident_form).
+//   - Else, and in what is left of those, rounds of at most two steps per device, which are bound by memory, with
+//     rounding to nearest even: stochastic rounding draws a second random block per pack and call (row walk
+//     -3 ... -5 %; resident with 24 and 32 devices -6 ... +2 %).  With more steps the row walk gains nothing (0 ... -3 %).
+bool light_round(const hadfl_handle *h, const RoundArgs &a) {
+  if (h->cfg.rounding == HADFL_ROUND_STOCHASTIC) return false;
+  for (int j = 0; j < a.n; ++j)
+    if (a.r[j].steps > kRowPerBlockMaxSteps) return false;
+  return true;
+}
+bool batchable(const hadfl_handle *h, const RoundArgs &a) {
   if (h->round_batch <= 1) return false;
   const size_t arena = arena_bytes(h);
   if (arena <= kBatchSmallArenaBytes) return true;
   if (arena > h->resident_arena_bytes && h->cfg.n_devices <= 16) return true;
-  if (h->cfg.rounding == HADFL_ROUND_STOCHASTIC) return false;
-  for (int i = 0; i < h->cfg.n_devices; ++i)
-    if (pl.row_steps[i] > kRowPerBlockMaxSteps) return false;
-  return true;
+  return light_round(h, a);
+}
+
+// How many of the collected rounds, from `first` on, go into the next launch: all, or, where a batch of all of them
+// does not gain, the light ones up to the next that is not, or a single round.
+int next_launch(const hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b, int first) {
+  const int left = b.n_rounds - first;
+  const size_t arena = arena_bytes(h);
+  if (left == 1 || arena <= kBatchSmallArenaBytes) return left;
+  if (arena <= h->resident_arena_bytes || h->cfg.n_devices > 16) return left;  // collected as light rounds only
+  if (first == 0 && resident_form(h, b)) return left;
+  int count = 0;
+  while (count < left && light_round(h, b.round[first + count])) ++count;
+  return count > 0 ? count : 1;
 }
 
 }  // namespace
@@ -1145,28 +1186,36 @@ int hadfl_rounds(hadfl_handle *h, int64_t first_round, int32_t n_rounds, const i
   // launch; the others are launched one by one.
   RoundBatch<kRoundBatchMax> batch;
   batch.n_rounds = 0;
-  uint32_t version_before[kMaxDevices];  // the counters before the pending batch, should its launch fail
-  uint64_t step_count_before[kMaxDevices];
+  uint32_t version_before[kRoundBatchMax][kMaxDevices];  // the counters before each pending round, should its launch fail
+  uint64_t step_count_before[kRoundBatchMax][kMaxDevices];
   auto flush = [&]() -> int {
-    if (batch.n_rounds == 0) return HADFL_OK;
-    int rc;
-    {
-      DeviceGuard guard(h->device);
-      if (batch.n_rounds == 1) {
-        RoundBatch<1> one;
-        one.n_rounds = 1;
-        one.round[0] = batch.round[0];
-        rc = launch_round(h, one, lr);
-      } else {
-        rc = launch_round(h, batch, lr);
+    int rc = HADFL_OK;
+    for (int first = 0; first < batch.n_rounds && rc == HADFL_OK;) {
+      const int count = next_launch(h, batch, first);
+      {
+        DeviceGuard guard(h->device);
+        if (count == 1) {
+          RoundBatch<1> one;
+          one.n_rounds = 1;
+          one.round[0] = batch.round[first];
+          rc = launch_round(h, one, lr);
+        } else if (count == batch.n_rounds) {
+          rc = launch_round(h, batch, lr);
+        } else {
+          RoundBatch<kRoundBatchMax> part;
+          part.n_rounds = count;
+          memcpy(part.round, batch.round + first, count * sizeof(RoundArgs));
+          rc = launch_round(h, part, lr);
+        }
       }
-    }
-    if (rc == HADFL_OK) {
-      h->stats_valid = true;
-      h->last_launch_rounds = batch.n_rounds;
-    } else {
-      memcpy(h->version, version_before, sizeof(version_before));
-      memcpy(h->step_count, step_count_before, sizeof(step_count_before));
+      if (rc == HADFL_OK) {
+        h->stats_valid = true;
+        h->last_launch_rounds = count;
+        first += count;
+      } else {
+        memcpy(h->version, version_before[first], sizeof(version_before[0]));
+        memcpy(h->step_count, step_count_before[first], sizeof(step_count_before[0]));
+      }
     }
     batch.n_rounds = 0;
     return rc;
@@ -1185,15 +1234,13 @@ int hadfl_rounds(hadfl_handle *h, int64_t first_round, int32_t n_rounds, const i
       rc = flush();
       if (rc == HADFL_OK) rc = round_by_separate_calls(h, ids, round_steps, N, lr, nullptr, k, sync, pl.sel);
     } else {
-      if (!batchable(h, pl)) rc = flush();
+      if (!batchable(h, pl.a)) rc = flush();
       if (rc == HADFL_OK) {
-        if (batch.n_rounds == 0) {
-          memcpy(version_before, h->version, sizeof(version_before));
-          memcpy(step_count_before, h->step_count, sizeof(step_count_before));
-        }
+        memcpy(version_before[batch.n_rounds], h->version, sizeof(version_before[0]));
+        memcpy(step_count_before[batch.n_rounds], h->step_count, sizeof(step_count_before[0]));
         batch.round[batch.n_rounds++] = pl.a;
         commit_round(h, pl, k, sync);
-        if (!batchable(h, pl) || batch.n_rounds >= h->round_batch) rc = flush();
+        if (!batchable(h, pl.a) || batch.n_rounds >= h->round_batch) rc = flush();
       }
     }
     if (rc != HADFL_OK) return rc;

@@ -11,7 +11,7 @@ import pytest
 import torch
 
 from gpu_common import require_gpu
-from paper_2111_08274_b200 import runtime, workloads
+from paper_2111_08274_b200 import binding, runtime, workloads
 from paper_2111_08274_b200.workloads import Workload
 
 pytestmark = pytest.mark.gpu
@@ -84,3 +84,36 @@ def test_small_arenas(n, P, k, hi):
 def test_more_chunks_than_blocks(n, k, beta):
     """16,384 blocks and chunks of 1024 parameters: each block has a second chunk, a few a third."""
     compare(n, 2 * 16_384 * 1024 + 5_003, k, tuple(1 + i % 2 for i in range(n)), "bf16_m16", beta, (3,), 1)
+
+
+@pytest.mark.parametrize("n,storage,per_round,launches", [
+    (16, "fp32", (8, 8), [1, 1]), (16, "fp32", (8,) * 8, [1] * 8), (16, "fp32", (1, 1, 8), [2, 1]),
+    (16, "fp32", (8, 1, 1, 1, 8), [1, 3, 1]), (16, "fp32", (1, 1, 5), [2, 1]), (16, "fp32", (1, 1, 5, 2), [4]),
+    (16, "fp32", (4, 3, 4, 4, 3, 4), [6]), (6, "fp32", (8, 8), [1, 1]), (6, "fp32", (8, 8, 8), [3]), (8, "fp32", (3, 3), [2]),
+    (16, "bf16", (8, 8), [1, 1]), (16, "bf16", (8, 8, 8), [3]), (14, "bf16", (8, 8), [2]),
+    (16, "bf16_m16_sr", (2, 2, 2, 2), [1] * 4), (16, "bf16_m16_sr", (1, 1), [2]), (14, "bf16_m16_sr", (8, 8, 8), [3])])
+def test_rounds_that_do_not_gain_are_launched_apart(n, storage, per_round, launches):
+    dtype, m_dtype, rounding, width = STORAGE[storage]
+    wl = Workload("apart", n, 166_000_000 // (n * width), 3, 1, "fixed", (1,) * n, grad_std=1e-2, dtype=dtype,
+                  m_dtype=m_dtype, rounding=rounding, seed=workloads.BASE_SEED + n)
+    batch, single = runtime.Arena(wl), runtime.Arena(wl)
+    steps = np.repeat(np.array(per_round, dtype=np.int32)[:, None], n, axis=1)
+    before = batch.h.launch_count()
+    got = batch.h.rounds(0, steps, wl.lr, wl.k, batch.select_seed, 2)
+    assert batch.h.launch_count() - before == len(launches)
+    stats = []
+    for r in range(len(steps)):
+        want = single.h.round(single.ids, steps[r], wl.lr, r, wl.k, single.select_seed, sync_all=r % 2 == 1)
+        assert np.array_equal(got[r], want)
+        stats.append(single.h.stats_read())
+    torch.cuda.synchronize()
+    assert torch.equal(batch.w, single.w) and torch.equal(batch.m, single.m)
+    assert all(np.array_equal(x, y) for x, y in zip(batch.h.get_versions(), single.h.get_versions()))
+    for back in range(launches[-1]):
+        for x, y in zip(batch.h.stats_read_round(back), stats[-1 - back]):
+            assert np.allclose(x, y, rtol=2.0 ** -23, atol=0)
+    with pytest.raises(binding.HadflError):
+        batch.h.stats_read_round(launches[-1])
+    batch.h.debug_check()
+    batch.close()
+    single.close()
