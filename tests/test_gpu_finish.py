@@ -1,9 +1,10 @@
 """The last-block finish of the statistics and of the fused round at the sizes where its loops change
 shape: block counts around the group size (128 blocks), around a warp's stride over the partial sums
 (32 lanes x 4 loads), one block, and more than one group; a launch with one round and one with several.
-The sums must match a double-precision sum over the arena as it stands afterwards.  Bound: a value is
-added to at most 8 others in a thread, then once across lanes and over 8 warps in fp32, all terms
-positive: relative error <= (8 + 1 + 8) * 2^-24 = 1.0e-6, and the output's own rounding 2^-24."""
+The sums must match a double-precision sum over the arena as it stands afterwards.  Bounds, all terms being
+positive: in the fused round a term is rounded at most 8 times in a thread's pack (each square is fused to the
+sum) and once across a pair of lanes, in the statistics kernel 16 times in a thread's chunk of 4 packs of 4;
+the rest is in fp64, and the output is rounded once more."""
 import numpy as np
 import pytest
 import torch
@@ -13,7 +14,7 @@ from paper_2111_08274_b200 import runtime, workloads
 from paper_2111_08274_b200.workloads import Workload
 
 pytestmark = pytest.mark.gpu
-BOUND = 18 * 2.0 ** -24
+ROUND, STATS = 10 * 2.0 ** -24, 17 * 2.0 ** -24
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -26,10 +27,10 @@ def sums(arena, ref):
     return (w * w).sum(1).cpu().numpy(), ((w - w[ref]) ** 2).sum(1).cpu().numpy()
 
 
-def check(got, want):
-    assert np.allclose(got[0], want[0], rtol=BOUND, atol=0)
+def check(got, want, bound):
+    assert np.allclose(got[0], want[0], rtol=bound, atol=0)
     # distances are sums over fp32 differences, each rounded once more before it is squared
-    assert np.allclose(got[1], want[1], rtol=BOUND + 2.0 ** -23, atol=0)
+    assert np.allclose(got[1], want[1], rtol=bound + 2.0 ** -23, atol=0)
 
 
 @pytest.mark.parametrize("blocks", [1, 2, 31, 32, 33, 127, 128, 129, 255, 257, 300])
@@ -39,9 +40,9 @@ def test_sums_over_block_counts(blocks, n, k, extra):
                   seed=workloads.BASE_SEED + blocks)
     arena = runtime.Arena(wl)
     sel = arena.run_round_fused(0)                       # a launch of one round
-    check(arena.h.stats_read(), sums(arena, int(sel[0])))
+    check(arena.h.stats_read(), sums(arena, int(sel[0])), ROUND)
     sel = arena.run_rounds_fused(1, 3)[-1]               # a launch of three
-    check(arena.h.stats_read(), sums(arena, int(sel[0])))
+    check(arena.h.stats_read(), sums(arena, int(sel[0])), ROUND)
     ref = n - 1
-    check(arena.h.stats(ref), sums(arena, ref))          # the statistics kernel
+    check(arena.h.stats(ref), sums(arena, ref), STATS)          # the statistics kernel
     arena.close()
