@@ -212,17 +212,30 @@ int hadfl_rounds(hadfl_handle *h, int64_t first_round, int32_t n_rounds, const i
 
 /* Rounds per launch.  Every operation of a round (Eq. 3, Eq. 5, the send to the other devices) is
  * elementwise in the parameter index, and the selections (Eq. 8) depend on versions the host knows
- * beforehand, so hadfl_rounds may hand several consecutive rounds to ONE launch of the fused kernel:
- * a block takes its columns through all of them before it moves to the next columns, and from the
- * second round on the replicas are read from L2 instead of HBM.  Results - parameters, momentum,
- * counters, selections - are those of the rounds launched one by one, bit for bit; so are every
- * round's statistics, except where the two launches take different forms of the kernel, which sum them
- * in different (equally fixed) orders: they then agree to rounding.  That is so for batches on large
- * fp32 arenas whose devices run at most 1.5 steps on average (packs of half the width), and for
- * n_devices * n_params <= 2^22 unless a launch of one round also takes the form for small vectors (at
- * most 2^17 parameters and n_devices * n_params <= 2^21).  hadfl_rounds batches the rounds that gain from it (every device runs at most two
- * steps and rounding is to nearest even, or the whole arena - parameters and momentum of all
- * devices - is at most 64 MiB) and launches the others singly.
+ * beforehand, so hadfl_rounds may hand several consecutive rounds to ONE launch: a block takes its
+ * columns through all of them before it moves to the next columns, and the replicas cross HBM once per
+ * launch.  The arena is the parameters and momentum of all devices; "large" is beyond 9/8 of the L2
+ * (142 MB with 126 MB).
+ * Which rounds share a launch:
+ *   - arenas of at most 64 MiB: all, whatever their steps and rounding;
+ *   - large arenas of at most 16 devices: batches of at most two steps per device on average with any number
+ *     of rounds, those with more steps from 2 to 6 rounds on, by devices, steps and storage (not at all with
+ *     more than 10 fp32 devices beyond four steps on average; stochastic rounding with 13 and 14 devices from
+ *     3 rounds on, with 15 and 16 from 6 on up to three steps, both from 2 on up to one and a half);
+ *   - else, and within batches that do not gain: neighbouring rounds in which no device runs more than two
+ *     steps, with rounding to nearest even.
+ * The other rounds are launched singly.
+ * Results - parameters, momentum, counters, selections - are those of the rounds launched one by one, bit
+ * for bit.  Statistics are bit for bit the same where both launches take the same form of the kernel, and
+ * agree to the rounding of their fp32 output where the forms, which sum in different (equally fixed)
+ * orders, are different ones.  The forms are:
+ *   - a warp per row: one round of at most 2^17 parameters and n_devices * n_params <= 2^21; several of
+ *     n_devices * n_params <= 2^22;
+ *   - the rows kept on the SM, several rounds only: other arenas of at most 64 MiB and 8 devices; large arenas
+ *     of at most 16 devices where the batch gains, as above; large arenas of more devices in batches of at
+ *     least 4 rounds of at most 1.5 steps on average, or of up to 24 devices in batches of at least 6;
+ *   - the walk over the rows: all else.  Of that, fp32 batches of at most 1.5 steps on average, with no device
+ *     beyond two, on arenas beyond 64 MiB of up to about 20 devices take packs of half the width, a third order.
  * hadfl_set_round_batch: the most rounds per launch, 1 .. 8 (default 8; 1 = never batch);
  * HADFL_ERR_INVALID outside that range.  hadfl_round_batch returns the setting (0 for NULL). */
 int hadfl_set_round_batch(hadfl_handle *h, int32_t max_rounds);
@@ -307,7 +320,9 @@ int hadfl_write_momentum(hadfl_handle *h, int32_t device_id, const float *src, i
 /* Model backup that overlaps with the rounds that follow (Section "Overall Design", item 9: the model
  * manager "regularly fetches the latest model").  hadfl_backup_begin takes a snapshot of the first
  * `count` parameters of device_id as they are at this point of the handle's stream (one device-to-
- * device copy on that stream into a staging row the library allocates on first use) and then moves
+ * device copy on that stream into a staging row the library allocates on first use, widened to fp32 on the
+ * way; where there is no room for that, bf16 rows are staged as they are and widened by the host in
+ * hadfl_backup_wait) and then moves
  * it to `dst` on a separate copy stream: the caller and the later work on the handle's stream do not
  * wait for the transfer.  dst (fp32, widened from bf16 storage) must stay valid until
  * hadfl_backup_wait returns, which blocks until the data has arrived; use pinned host memory for the
