@@ -362,6 +362,9 @@ int launch_local_step(hadfl_handle *h, const LocalStepArgs &a, float lr) {
 //   one round per launch: 8 devices 131,072: 12.7 / 12.0, 28.8 / 17.8; 200,000: 12.7 / 14.7, 29.1 / 22.9;
 //     16 devices 65,536: 18.0 / 12.4, 51.3 / 18.8; 131,072: 18.6 / 17.9, 51.6 / 28.8; 262,144: 18.8 / 26.8;
 //     32 devices 131,072 (16 selected): 31.1 / 37.2
+//   stochastic rounding (bf16 parameters and momentum; these builds spill 60 to 70 bytes a thread), one round: 8
+//     devices 131,072: 22.5 / 14.0, 23.7 / 17.3 (uniform 1..8); 16 devices 131,072: 24.7 / 20.5, 41.8 / 28.2; 8 rounds:
+//     16 devices 262,144: 26.9 / 20.4, 45.1 / 34.8; 32 devices 131,072: 46.0 / 26.8, 86.6 / 44.3
 bool rows_form(const hadfl_handle *h, int n_rounds) {
   const int64_t P = h->cfg.n_params, work = h->cfg.n_devices * P;
   return n_rounds > 1 ? work <= ((int64_t)1 << 22) : P <= ((int64_t)1 << 17) && work <= ((int64_t)1 << 21);
@@ -382,7 +385,7 @@ int allow_all_shared(hadfl_handle *h, Kernel kernel, bool &done) {
   return HADFL_OK;
 }
 
-// Rows form: tiles of a block (at least 8 warps) and blocks of a launch.
+// Rows form: tiles of a block (as many as make up to 8 warps, or one) and blocks of a launch.
 int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
 int64_t rows_grid(int n_devices, int64_t n_params) {
   constexpr int kCols = 32 * StepPack<float>::E;

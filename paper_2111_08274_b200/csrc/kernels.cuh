@@ -1537,7 +1537,8 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 // Values move between the arena and the SM as they are: NaNs of rows that nothing changes keep their bits.
 // ------------------------------------------------------------------------------------------
 constexpr int kResidentThreads = 128;
-constexpr int kResidentMaxBlocks = 6;  // per SM, by registers (80 a thread); shared memory sets the actual number
+constexpr int kResidentMaxBlocks = 6;  // per SM: what the registers are bounded for (80 a thread; builds that use no more
+                                       // than 72 could have 7); shared memory sets the actual number
 
 struct ResidentBatch {
   int32_t n, k, n_rounds;
