@@ -1521,7 +1521,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 //
 // What bounds it: on large vectors the row walk through L2 ran into the board's power cap (1000 W, SM clock
 // down to 1600 - 1750 MHz); here a round moves a fraction of the bytes, keeps the full clock at 500 - 900 W
-// and is bound by instruction latency at 3 to 6 warps per scheduler (232 instructions per row and pack).
+// and is bound by instruction latency at 3 to 6 warps per scheduler (237 instructions per row and pack at one step).
 // How many blocks share an SM decides between warps to hide latency with and rows that find room (the
 // host chooses).  Sustained, us per round of a batch of 8, row walk -> resident: 16 devices, 2^24, one
 // step 496 -> 409 (before the 32-byte stores 3, 4, 5, 6 blocks: 424, 436, 431, 478), two steps at 14.7 M 635 -> 534 (574, 556, 534,
