@@ -585,27 +585,59 @@ __device__ __forceinline__ void sgd_steps(float (&w)[4 * NB], float (&m)[4 * NB]
 // group takes the low half of word `lane` for its parameter and the high half for its momentum.
 // The result is exactly representable in bf16, so the conversion at the store changes nothing.
 // ------------------------------------------------------------------------------------------
+// What bounds it is instructions: one more generator block per group (the first round's products are the
+// gradients' own), then the values.  One test per pack finds out whether any of its values is not finite, where
+// a test and a conversion per value stood, and what has been rounded here is not rounded again on its way to
+// the aggregate.  Measured, us per round: 16 devices, 33.5 M parameters, steps 1,1,2,2,4,4,8,8, bf16
+// throughout 2346 -> 2238; a batch of 8, 8 devices, 16.8 M, one step 301 -> 281.5.
 __device__ __forceinline__ float bf16_stochastic(float v, uint32_t r16) {
-  const uint32_t bits = __float_as_uint(v);
-  if ((bits & 0x7F800000u) == 0x7F800000u) return __bfloat162float(__float2bfloat16_rn(v));
-  return __uint_as_float((bits + r16) & 0xFFFF0000u);
+  return __uint_as_float((__float_as_uint(v) + r16) & 0xFFFF0000u);
+}
+__device__ __forceinline__ float bf16_stochastic_any(float v, uint32_t r16) {
+  if ((__float_as_uint(v) & 0x7F800000u) == 0x7F800000u) return __bfloat162float(__float2bfloat16_rn(v));
+  return bf16_stochastic(v, r16);
+}
+// The larger magnitude, NaN if either is.
+__device__ __forceinline__ float max_magnitude(float a, float b) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(fabsf(a)), "f"(fabsf(b)));
+  return m;
 }
 
 template <typename MT, int NB>
-__device__ __forceinline__ void round_stochastic(float (&w)[4 * NB], float (&m)[4 * NB], int64_t pack,
+__device__ __forceinline__ void round_stochastic(float (&w)[4 * NB], float (&m)[4 * NB], const GroupProducts<NB> &gp,
                                                  const RowStep &rs, const PhiloxKeys &keys) {
+  constexpr int E = 4 * NB;
+  uint32_t x[NB][4];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    uint32_t x0 = (uint32_t)(pack * NB + b);
-    uint32_t x1 = rs.base_lo + (uint32_t)rs.steps - 1u;
-    uint32_t x2 = (uint32_t)rs.row;
-    uint32_t x3 = rs.r1_c2 ^ keys.b[0] ^ (kTagGrad ^ kTagRound);  // tag | high bits of the step index
-    philox4x32_10(x0, x1, x2, x3, keys);
-    const uint32_t x[4] = {x0, x1, x2, x3};
+    x[b][0] = rs.r1_c0 ^ (rs.base_lo + (uint32_t)rs.steps - 1u);
+    x[b][1] = rs.r1_c1;
+    x[b][2] = gp.hi[b] ^ rs.r1_c2 ^ (kTagGrad ^ kTagRound);
+    x[b][3] = gp.lo[b];
+  }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      w[4 * b + i] = bf16_stochastic(w[4 * b + i], x[i] & 0xFFFFu);
-      if (sizeof(MT) == 2) m[4 * b + i] = bf16_stochastic(m[4 * b + i], x[i] >> 16);
+  for (int r = 1; r < 10; ++r)
+#pragma unroll
+    for (int b = 0; b < NB; ++b) philox_round(x[b][0], x[b][1], x[b][2], x[b][3], keys.a[r], keys.b[r]);
+  float largest = max_magnitude(w[0], w[1]);
+#pragma unroll
+  for (int i = 2; i < E; ++i) largest = max_magnitude(largest, w[i]);
+  if (sizeof(MT) == 2) {
+#pragma unroll
+    for (int i = 0; i < E; ++i) largest = max_magnitude(largest, m[i]);
+  }
+  if (largest < __uint_as_float(0x7F800000u)) {
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      w[i] = bf16_stochastic(w[i], x[i / 4][i % 4] & 0xFFFFu);
+      if (sizeof(MT) == 2) m[i] = bf16_stochastic(m[i], x[i / 4][i % 4] >> 16);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      w[i] = bf16_stochastic_any(w[i], x[i / 4][i % 4] & 0xFFFFu);
+      if (sizeof(MT) == 2) m[i] = bf16_stochastic_any(m[i], x[i / 4][i % 4] >> 16);
     }
   }
 }
@@ -641,7 +673,7 @@ k_local_step(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, LocalStep
     };
     auto body = [&](int j, float (&wv)[E], float (&mv)[E]) {
       sgd_steps<Gen, E / 4>(wv, mv, gp, a.r[j], keys, k);
-      if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, a.r[j], keys);
+      if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, gp, a.r[j], keys);
       st_pack_any(at_row<WT>(wp, a.r[j].w_off), 0, live, wv);
       st_pack_any(at_row<MT>(mp, a.r[j].m_off), 0, live, mv);
     };
@@ -1190,10 +1222,12 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
             unpack(rw, wv);
             unpack(rm, mv);
             sgd_steps<Gen, E / 4>(wv, mv, gp, a.r[j], keys, k);
-            if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, a.r[j], keys);
+            if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, gp, a.r[j], keys);
             st_pack_any(at_row<MT>(mp, a.r[j].m_off), 0, live, mv);
+            if constexpr (RM == 0) {
 #pragma unroll
-            for (int i = 0; i < E; ++i) wv[i] = as_stored(wv[i], w);
+              for (int i = 0; i < E; ++i) wv[i] = as_stored(wv[i], w);
+            }
             if (live < E) {  // the ragged last pack of a row and the lanes beyond it: dead lanes stay 0
 #pragma unroll
               for (int i = 0; i < E; ++i) wv[i] = i < live ? wv[i] : 0.f;
@@ -1423,11 +1457,14 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
         const int j = st.visit, write_all = b.write_all[r];
         if (rs.steps > 0) {
           sgd_steps<Gen, E / 4>(wv, mv, gp, rs, keys, k);
-          if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, rs, keys);
+          if constexpr (RM == 1) {
+            round_stochastic<MT, E / 4>(wv, mv, gp, rs, keys);
+          } else {
 #pragma unroll
-          for (int i = 0; i < E; ++i) {
-            wv[i] = as_stored(wv[i], w);
-            mv[i] = as_stored(mv[i], m);
+            for (int i = 0; i < E; ++i) {
+              wv[i] = as_stored(wv[i], w);
+              mv[i] = as_stored(mv[i], m);
+            }
           }
           if (live < E) {  // lanes beyond the end of the vector stay 0 in the sums
 #pragma unroll
@@ -1785,7 +1822,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
               step_noise<Gen, E / 4>(nz, e, c2_first, gp, rs, keys, k);
               step_update<E / 4>(wv, mv, nz, k);
             }
-            if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, p, rs, keys);
+            if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, gp, rs, keys);
             pack_raw(wv, rw);
             store_w(where, row, rw);
             pack_raw(mv, rm);

@@ -202,3 +202,36 @@ def test_written_momentum_is_rounded_and_options_need_bf16_parameters(oracle):
         with pytest.raises(binding.HadflError) as e:
             binding.Hadfl(2, 64, **kw)
         assert e.value.code == binding.ERR_INVALID
+
+
+@pytest.mark.parametrize("m_dtype", [0, 1])
+@pytest.mark.parametrize("form", ["local", "rows", "walk", "on_sm"])
+def test_values_that_are_not_finite_beside_finite_ones(oracle, form, m_dtype):
+    """A pack of 8 is tested as a whole for infinities and NaNs, which are rounded to nearest even; the finite
+    values beside them keep their random bits.  In the parameters, in the momentum, at a pack's first and last
+    place, in the ragged last pack, and values that the rounding itself may carry to infinity."""
+    n, P, rounds = {"local": (3, 4099, 1), "rows": (4, 1003, 2), "walk": (4, 140_003, 1), "on_sm": (3, 1_500_003, 2)}[form]
+    wl = wl_of(n, P, m_dtype, 1, grad_std=0.0, weight_decay=0.3, momentum=0.9, k=1)
+    h, sim = binding.Hadfl.from_workload(wl), make_sim(oracle, wl)
+    rows = workloads.random_rows(n, P, seed=31)
+    mom = workloads.random_rows(n, P, seed=32, std=0.01)
+    big = np.float32(3.38e38)
+    for i, (at, v) in enumerate([(0, np.inf), (15, np.nan), (17, -np.inf), (31, big), (P - 1, np.nan), (P - 2, -big)]):
+        rows[i % n, at] = v
+        mom[(i + 1) % n, at + 8 if at < 32 else at] = v
+    load_rows(h, sim, rows, mom)
+    steps = np.tile(np.array([1 + i for i in range(n)], dtype=np.int32), (rounds, 1))
+    if form == "local":
+        h.local_step(range(n), steps[0], 0.05)
+    else:
+        sel = h.rounds(0, steps, 0.05, 1, 9)
+    for r in range(rounds):
+        sim.local_step(list(range(n)), steps[r], 0.05)
+        if form != "local":
+            want = sim.select(r, 1, 9)
+            assert np.array_equal(sel[r], want)
+            sim.aggregate(want)
+    for i in range(n):
+        assert np.array_equal(h.read_params(i), sim.read_params(i), equal_nan=True), i
+        assert np.array_equal(h.read_momentum(i), sim.read_momentum(i), equal_nan=True), i
+    h.destroy()
