@@ -32,7 +32,7 @@ struct hadfl_handle {
   size_t smem_per_sm = 0;
   int smem_per_block = 0;                   // most shared memory of a block, static and dynamic
   bool rows_smem[2] = {};                   // allow_all_shared is done for k_round_rows (launches of one round, batches)
-  bool resident_smem[2] = {};               // ... for k_rounds_resident (a part of the rows on the SM, all of them)
+  bool resident_smem[3] = {};               // ... for the builds of k_rounds_resident
   size_t resident_arena_bytes = 0;  // batches on arenas beyond this are resident on the SMs
   PhiloxKeys keys;
   uint32_t version[kMaxDevices];
@@ -529,16 +529,24 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
       if (rows_on_chip(blocks_per_sm) < rows_on_chip(blocks_per_sm - 1)) --blocks_per_sm;
       while (blocks_per_sm > 2 && in_l2(blocks_per_sm) > 0.55 * h->l2_bytes) --blocks_per_sm;
     }
+    // one visit per row and round: fp32, up to 1.5 steps per device on average (measured at Resident::kPartOneVisit)
+    const bool one_visit = sizeof(WT) == 4 && rows_on_chip(blocks_per_sm) < n && mean_steps_x2 <= 3;
+    const int max_blocks = one_visit ? kResidentOneVisitMaxBlocks : kResidentMaxBlocks;
+    if (blocks_per_sm > max_blocks) blocks_per_sm = max_blocks;
     q.n_on_chip = rows_on_chip(blocks_per_sm);
     // As much shared memory as keeps the number of blocks at that.
     size_t smem = q.n_on_chip * kRowBytes + sums;
     const size_t floor_bytes = h->smem_per_sm / (blocks_per_sm + 1) - kSmemReserve + 1024;
-    if (smem < floor_bytes && blocks_per_sm < kResidentMaxBlocks) smem = floor_bytes;
+    if (smem < floor_bytes && blocks_per_sm < max_blocks) smem = floor_bytes;
     const int64_t chunks = (h->cfg.n_params + 8 * kResidentThreads - 1) / (8 * kResidentThreads);
     const int grid = (int)(chunks < kRoundGridCap ? chunks : kRoundGridCap);
-    auto kernel = q.n_on_chip == n ? k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, true>
-                                   : k_rounds_resident<WT, MT, NormalsFast, decltype(rm)::value, false>;
-    const int rc = allow_all_shared(h, kernel, h->resident_smem[q.n_on_chip == n]);
+    constexpr int RM = decltype(rm)::value;
+    const Resident form = q.n_on_chip == n ? Resident::kAll : one_visit ? Resident::kPartOneVisit : Resident::kPart;
+    auto kernel = form == Resident::kAll ? k_rounds_resident<WT, MT, NormalsFast, RM, Resident::kAll>
+                                         : k_rounds_resident<WT, MT, NormalsFast, RM, Resident::kPart>;
+    if constexpr (sizeof(WT) == 4)
+      if (form == Resident::kPartOneVisit) kernel = k_rounds_resident<WT, MT, NormalsFast, RM, Resident::kPartOneVisit>;
+    const int rc = allow_all_shared(h, kernel, h->resident_smem[(int)form]);
     if (rc != HADFL_OK) return rc;
     kernel<<<grid, kResidentThreads, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->cfg.n_params, h->keys,
                                                         step_consts(h, lr), scratch, q);

@@ -1578,6 +1578,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 constexpr int kResidentThreads = 128;
 constexpr int kResidentMaxBlocks = 6;  // per SM: what the registers are bounded for (80 a thread; builds that use no more
                                        // than 72 could have 7); shared memory sets the actual number
+constexpr int kResidentOneVisitMaxBlocks = 5;  // ... of the build with one visit per row and round
 
 struct ResidentBatch {
   int32_t n, k, n_rounds;
@@ -1680,11 +1681,26 @@ constexpr size_t resident_sums_bytes(int n, int rounds) {
   return (kResidentThreads / 32) * (sizeof(double) * 2 * n * rounds + sizeof(float) * WarpRowSums::kFloats);
 }
 
-template <typename WT, typename MT, typename Gen, int RM, bool kAllOnChip>
-__global__ void __launch_bounds__(kResidentThreads, kResidentMaxBlocks)
+// The builds of the kernel: all rows on the SM; a part of them; a part of them, and one visit per row and round.
+// With visits apart - steps of all rows, aggregation, sums - a row that lives in L2 crosses to the SM and back up to
+// three times a round; with one, in draw order, once, and a selected row is stored only as the aggregate, but the
+// aggregate and the row's sums then take registers through the steps: with several steps per row, where warps to
+// hide latency with count for more, or with all rows on the SM, that costs more than it saves.  Sustained, us per
+// round of a batch of 8, apart / one visit: 16 devices, 2^24, one step 406 / 387, 2^22 112.4 / 107.3; 32 devices,
+// 2^22 300 / 282; 16 devices, 2^24, two steps 590 / 587; 14.7 M, steps 1,1,2,2,4,4,8,8 809 / 831; all rows on the SM, 8
+// devices, 11.2 M, one step 118 / 121; bf16 parameters, 16 devices, 2^22, one step 102 / 107.  With 6 blocks per SM
+// instead of 5: 2^24, one step 397.
+enum class Resident { kAll, kPart, kPartOneVisit };
+constexpr int resident_max_blocks(Resident form) {
+  return form == Resident::kPartOneVisit ? kResidentOneVisitMaxBlocks : kResidentMaxBlocks;
+}
+
+template <typename WT, typename MT, typename Gen, int RM, Resident kForm>
+__global__ void __launch_bounds__(kResidentThreads, resident_max_blocks(kForm))
 k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, PhiloxKeys keys,
                   StepConsts k, RoundScratch scratch, const __grid_constant__ ResidentBatch b) {
   constexpr int E = 8, kWarps = kResidentThreads / 32;
+  constexpr bool kAllOnChip = kForm == Resident::kAll;
   constexpr int kWords = E * (int)sizeof(MT) / 4;  // tensor memory columns per row
   using Store = RowStore<WT>;
   using Sums = WarpRowSums;
@@ -1791,11 +1807,11 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
 #pragma unroll 1
       for (int r = 0; r < b.n_rounds; ++r) {
         double *line = lines + (warp * b.n_rounds + r) * 2 * n;
-        // ---- local steps
-        const int n_step = b.n_stepping[r];
-#pragma unroll 1
-        for (int j = 0; j < n_step; ++j) {
-          const int row = b.order[r][j];
+        const int write_all = b.write_all[r];
+        float acc[E];
+        int slot = 0;
+        // The steps of a row, from where it lives to registers; the momentum goes back at once.
+        auto steps_of = [&](auto where, int row, float (&wv)[E]) {
           RowStep rs;
           rs.row = row;
           rs.steps = b.s[r][row].steps;
@@ -1806,97 +1822,163 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
           uint32_t c2_first[E / 4];
 #pragma unroll
           for (int g = 0; g < E / 4; ++g) c2_first[g] = gp.hi[g] ^ rs.r1_c2;
-          at_place(row, [&](auto where, int row) {
-            float wv[E], mv[E];
-            RawPack<WT, E> rw;
-            RawPack<MT, E> rm;
-            load_m(where, row, rm);
-            load_w(where, row, rw);
-            // the values are on their way while the first step's noise is drawn
-            float2 nz[E / 4][2];
-            step_noise<Gen, E / 4>(nz, 0, c2_first, gp, rs, keys, k);
-            m_arrived(where, rm);
-            unpack(rm, mv);
-            unpack(rw, wv);
-            step_update<E / 4>(wv, mv, nz, k);
+          float mv[E];
+          RawPack<WT, E> rw;
+          RawPack<MT, E> rm;
+          load_m(where, row, rm);
+          load_w(where, row, rw);
+          // the values are on their way while the first step's noise is drawn
+          float2 nz[E / 4][2];
+          step_noise<Gen, E / 4>(nz, 0, c2_first, gp, rs, keys, k);
+          m_arrived(where, rm);
+          unpack(rm, mv);
+          unpack(rw, wv);
+          step_update<E / 4>(wv, mv, nz, k);
 #pragma unroll 1
-            for (int e = 1; e < rs.steps; ++e) {
-              step_noise<Gen, E / 4>(nz, e, c2_first, gp, rs, keys, k);
-              step_update<E / 4>(wv, mv, nz, k);
-            }
-            if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, gp, rs, keys);
-            pack_raw(wv, rw);
-            store_w(where, row, rw);
-            pack_raw(mv, rm);
-            store_m(where, row, rm);
-          });
-        }
-        // ---- aggregation with write-back: acc = a_0 w_0, then acc = fma(a_j, w_j, acc) in draw order
-        float acc[E];
-        at_place(b.draw[r][0], [&](auto where, int row) {
-          float wv[E];
-          values(where, row, wv);
+          for (int e = 1; e < rs.steps; ++e) {
+            step_noise<Gen, E / 4>(nz, e, c2_first, gp, rs, keys, k);
+            step_update<E / 4>(wv, mv, nz, k);
+          }
+          if constexpr (RM == 1) round_stochastic<MT, E / 4>(wv, mv, gp, rs, keys);
+          pack_raw(mv, rm);
+          store_m(where, row, rm);
+        };
+        // Aggregation in draw order: acc = a_0 w_0, then acc = fma(a_j, w_j, acc)
+        auto start_aggregate = [&](const float (&wv)[E]) {
           const float a0 = b.a[r][0];
 #pragma unroll
           for (int i = 0; i < E; ++i) acc[i] = __fmul_rn(a0, wv[i]);
-        });
-#pragma unroll 1
-        for (int j = 1; j < n_sel; ++j)
-          at_place(b.draw[r][j], [&](auto where, int row) {
-            float wv[E];
-            values(where, row, wv);
-            const float aj = b.a[r][j];
+        };
+        auto add_selected = [&](int j, const float (&wv)[E]) {
+          const float aj = b.a[r][j];
 #pragma unroll
-            for (int i = 0; i < E; ++i) acc[i] = fmaf(aj, wv[i], acc[i]);
-          });
-        float n2 = 0.f;
+          for (int i = 0; i < E; ++i) acc[i] = fmaf(aj, wv[i], acc[i]);
+        };
+        // The aggregate goes to the first n_holders devices of the draw.
+        auto hand_out = [&](int n_holders) {
+          float n2 = 0.f;
 #pragma unroll
-        for (int i = 0; i < E; ++i) {
-          acc[i] = as_stored(acc[i], w);
-          n2 = fmaf(acc[i], acc[i], n2);
-        }
-        const int write_all = b.write_all[r], n_holders = write_all == 1 ? n : n_sel;
-        float d2_held = 0.f;  // of the devices that are overwritten: as (acc - acc)^2, NaN where acc is not finite
-        if (write_all == 1) {
+          for (int i = 0; i < E; ++i) {
+            acc[i] = as_stored(acc[i], w);
+            n2 = fmaf(acc[i], acc[i], n2);
+          }
+          float d2_held = 0.f;  // of the devices that are overwritten: as (acc - acc)^2, NaN where acc is not finite
+          if (write_all == 1) {
 #pragma unroll
-          for (int i = 0; i < E; ++i) d2_held = fmaf(acc[i], 0.f, d2_held);
-        }
-        {
+            for (int i = 0; i < E; ++i) d2_held = fmaf(acc[i], 0.f, d2_held);
+          }
           RawPack<WT, E> ra;
           pack_raw(acc, ra);
 #pragma unroll 1
           for (int t = b.first_store[r]; t < n_holders; ++t)
             at_place(b.draw[r][t], [&](auto where, int row) { store_w(where, row, ra); });
-        }
-        Sums::add(slots, 0, n2, d2_held, lane);  // one value for all holders
-        // ---- the other devices: keep their own model, or mix the aggregate into it
-        int slot = 0;
-#pragma unroll 1
-        for (int j = n_holders; j < n; ++j) {
-          float s2 = 0.f, d2 = 0.f;
-          at_place(b.draw[r][j], [&](auto where, int row) {
-            float wv[E];
-            values(where, row, wv);
-            if (write_all) {
+          Sums::add(slots, 0, n2, d2_held, lane);  // one value for all holders
+        };
+        auto mix = [&](float (&wv)[E]) {
 #pragma unroll
-              for (int i = 0; i < E; ++i)
-                wv[i] = as_stored(fmaf(b.beta, acc[i], __fmul_rn(b.one_minus_beta, wv[i])), w);
-              RawPack<WT, E> rw;
-              pack_raw(wv, rw);
-              store_w(where, row, rw);
-            }
-#pragma unroll
-            for (int i = 0; i < E; ++i) {
-              const float d = wv[i] - acc[i];
-              s2 = fmaf(wv[i], wv[i], s2);
-              d2 = fmaf(d, d, d2);
-            }
-          });
+          for (int i = 0; i < E; ++i)
+            wv[i] = as_stored(fmaf(b.beta, acc[i], __fmul_rn(b.one_minus_beta, wv[i])), w);
+        };
+        auto add_sums = [&](int j, float s2, float d2) {
           if (++slot == Sums::kRows) {
             Sums::fold(slots, j - Sums::kRows, Sums::kRows, line, lane);
             slot = 0;
           }
           Sums::add(slots, slot, s2, d2, lane);
+        };
+        auto row_sums = [&](const float (&wv)[E], float &s2, float &d2) {
+          s2 = d2 = 0.f;
+#pragma unroll
+          for (int i = 0; i < E; ++i) {
+            const float d = wv[i] - acc[i];
+            s2 = fmaf(wv[i], wv[i], s2);
+            d2 = fmaf(d, d, d2);
+          }
+        };
+        if constexpr (kForm == Resident::kPartOneVisit) {
+#pragma unroll
+          for (int i = 0; i < E; ++i) acc[i] = -0.f;  // fma(a, w, -0) is a w, whatever its sign
+#pragma unroll 1
+          for (int j = 0; j < n; ++j)
+            at_place(b.draw[r][j], [&](auto where, int row) {
+              float wv[E];
+              const bool stepped = b.s[r][row].steps > 0;
+              if (stepped) {
+                steps_of(where, row, wv);
+#pragma unroll
+                for (int i = 0; i < E; ++i) wv[i] = as_stored(wv[i], w);
+                if (live < E) {
+#pragma unroll
+                  for (int i = 0; i < E; ++i) wv[i] = i < live ? wv[i] : 0.f;
+                }
+              } else {
+                values(where, row, wv);
+              }
+              if (j < n_sel) {
+                add_selected(j, wv);
+                if (j == n_sel - 1) hand_out(n_sel);
+              } else {
+                if (write_all == 2) mix(wv);
+                if (write_all == 1) {
+#pragma unroll
+                  for (int i = 0; i < E; ++i) wv[i] = acc[i];
+                }
+                if (stepped || write_all) {
+                  RawPack<WT, E> rw;
+                  pack_raw(wv, rw);
+                  store_w(where, row, rw);
+                }
+                if (write_all != 1) {
+                  float s2, d2;
+                  row_sums(wv, s2, d2);
+                  add_sums(j, s2, d2);
+                }
+              }
+            });
+        } else {
+          // ---- local steps
+          const int n_step = b.n_stepping[r];
+#pragma unroll 1
+          for (int j = 0; j < n_step; ++j)
+            at_place(b.order[r][j], [&](auto where, int row) {
+              float wv[E];
+              steps_of(where, row, wv);
+              RawPack<WT, E> rw;
+              pack_raw(wv, rw);
+              store_w(where, row, rw);
+            });
+          // ---- aggregation with write-back
+          at_place(b.draw[r][0], [&](auto where, int row) {
+            float wv[E];
+            values(where, row, wv);
+            start_aggregate(wv);
+          });
+#pragma unroll 1
+          for (int j = 1; j < n_sel; ++j)
+            at_place(b.draw[r][j], [&](auto where, int row) {
+              float wv[E];
+              values(where, row, wv);
+              add_selected(j, wv);
+            });
+          const int n_holders = write_all == 1 ? n : n_sel;
+          hand_out(n_holders);
+          // ---- the other devices: keep their own model, or mix the aggregate into it
+#pragma unroll 1
+          for (int j = n_holders; j < n; ++j) {
+            float s2, d2;
+            at_place(b.draw[r][j], [&](auto where, int row) {
+              float wv[E];
+              values(where, row, wv);
+              if (write_all) {
+                mix(wv);
+                RawPack<WT, E> rw;
+                pack_raw(wv, rw);
+                store_w(where, row, rw);
+              }
+              row_sums(wv, s2, d2);
+            });
+            add_sums(j, s2, d2);
+          }
         }
         Sums::fold(slots, write_all == 1 ? n_sel - 1 : n - 1 - slot, slot + 1, line, lane);
         tmem_wait_store();
