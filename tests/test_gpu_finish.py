@@ -46,3 +46,14 @@ def test_sums_over_block_counts(blocks, n, k, extra):
     ref = n - 1
     check(arena.h.stats(ref), sums(arena, ref), STATS)          # the statistics kernel
     arena.close()
+
+
+@pytest.mark.parametrize("blocks,rounds", [(481, 1), (482, 1), (160, 3), (161, 3)])
+def test_one_group_and_several(blocks, rounds):
+    """17 devices: 34 sums per round and block on both sides of the 16,384 that one block adds alone."""
+    wl = Workload("fin", 17, 2048 * blocks - 1, 5, 1, "fixed", (1,) * 17, grad_std=1e-2, seed=workloads.BASE_SEED + blocks)
+    arena = runtime.Arena(wl)
+    for first in (0, rounds):                            # the tickets are back at zero for the second launch
+        sel = arena.run_rounds_fused(first, rounds)[-1]
+        check(arena.h.stats_read(), sums(arena, int(sel[0])), ROUND)
+    arena.close()
