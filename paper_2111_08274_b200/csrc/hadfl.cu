@@ -31,7 +31,7 @@ struct hadfl_handle {
   int l2_bytes = 0;
   size_t smem_per_sm = 0;
   int smem_per_block = 0;                   // most shared memory of a block, static and dynamic
-  bool rows_smem[2] = {};                   // allow_all_shared is done for k_round_rows (launches of one round, batches)
+  bool rows_smem[3] = {};                   // allow_all_shared is done for k_round_rows (one round, batches, batches of a block per SM)
   bool resident_smem[3] = {};               // ... for the builds of k_rounds_resident
   size_t resident_arena_bytes = 0;  // batches on arenas beyond this are resident on the SMs
   PhiloxKeys keys;
@@ -385,13 +385,24 @@ int allow_all_shared(hadfl_handle *h, Kernel kernel, bool &done) {
   return HADFL_OK;
 }
 
-// Rows form: tiles of a block (as many as make up to 8 warps, or one) and blocks of a launch.
-int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
-int64_t rows_grid(int n_devices, int64_t n_params) {
+// Rows form: tiles of a block, as many as make up to 8 warps, or one, and blocks of a launch.
+int64_t rows_tiles(int64_t n_params) {
   constexpr int kCols = 32 * StepPack<float>::E;
-  const int64_t tiles = (n_params + kCols - 1) / kCols;
-  const int64_t blocks = (tiles + rows_groups(n_devices) - 1) / rows_groups(n_devices);
+  return (n_params + kCols - 1) / kCols;
+}
+int64_t rows_grid(int64_t n_params, int groups) {
+  const int64_t blocks = (rows_tiles(n_params) + groups - 1) / groups;
   return blocks < kRowsGridCap ? blocks : kRowsGridCap;
+}
+int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
+// Batches: where blocks of up to 16 warps leave no SM with two of them, as few tiles per block as do that (0: they do
+// not): the slowest SM then has fewer warps to run, and every warp can have twice the registers.  Such a block gets
+// all 16 warps, for the finish.  Measured, us per round of a batch of 8, tiles for 8 warps / one block per SM / the same
+// without the warps for the finish: 4 devices, 100,000 parameters 3.54 / 2.83 / 2.95, 30,000 2.72 / 2.10 / 2.65; 2 devices,
+// 300,001 2.53 / 2.12 / 2.12, 30,000 1.78 / 1.42 / 2.07; 8 devices, 70,001 4.88 / 4.25; 16 devices, 37,000 5.38 / 5.17.
+int rows_groups_one_per_sm(const hadfl_handle *h) {
+  const int64_t most = kRowsFewThreads / 32 / h->cfg.n_devices, tiles = rows_tiles(h->cfg.n_params);
+  return tiles <= h->sm_count * (most < 8 ? most : 8) ? (int)((tiles + h->sm_count - 1) / h->sm_count) : 0;
 }
 
 template <int NR>
@@ -404,7 +415,8 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
     q.n = h->cfg.n_devices;
     q.k = b.round[0].k;
     q.n_rounds = b.n_rounds;
-    q.groups = rows_groups(q.n);
+    const int few = NR > 1 ? rows_groups_one_per_sm(h) : 0;
+    q.groups = few ? few : rows_groups(q.n);
     q.beta = b.round[0].beta;
     q.one_minus_beta = b.round[0].one_minus_beta;
     for (int r = 0; r < b.n_rounds; ++r) {
@@ -413,13 +425,16 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
       memcpy(q.a[r], a.a, sizeof(a.a));
       for (int j = 0; j < q.n; ++j) q.s[r][a.r[j].row] = RowsStep{a.r[j].steps, a.r[j].base_lo, a.r[j].r1_c2, j};
     }
-    const int grid = (int)rows_grid(q.n, h->cfg.n_params);
+    const int grid = (int)rows_grid(h->cfg.n_params, q.groups);
     const size_t smem = rows_shared_bytes<WT, E>(q.groups, q.n, q.k, b.n_rounds);
-    auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR>;
-    const int rc = allow_all_shared(h, kernel, h->rows_smem[NR > 1]);
+    auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR, kRowsMaxThreads>;
+    if constexpr (NR > 1)
+      if (few) kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR, kRowsFewThreads>;
+    const int rc = allow_all_shared(h, kernel, h->rows_smem[few ? 2 : NR > 1]);
     if (rc != HADFL_OK) return rc;
-    kernel<<<grid, q.groups * q.n * 32, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->stride, h->cfg.n_params, h->keys,
-                                                           step_consts(h, lr), scratch, q);
+    const int threads = few ? kRowsFewThreads : q.groups * q.n * 32;
+    kernel<<<grid, threads, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->stride, h->cfg.n_params, h->keys,
+                                               step_consts(h, lr), scratch, q);
     h->last_launch_pack = E;
     return check_launch(h);
   });
@@ -806,8 +821,7 @@ int hadfl_init(const hadfl_config *cfg, hadfl_handle **out) {
                           (size_t)cfg->n_devices * (size_t)cfg->n_params * 8 > kBatchSmallArenaBytes;
   }
   int scratch_grid = h->round_grid_half_packs > h->round_grid ? h->round_grid_half_packs : h->round_grid;
-  if (rows_grid(cfg->n_devices, cfg->n_params) > scratch_grid)
-    scratch_grid = (int)rows_grid(cfg->n_devices, cfg->n_params);
+  if (rows_grid(cfg->n_params, 1) > scratch_grid) scratch_grid = (int)rows_grid(cfg->n_params, 1);
   const size_t n_groups = (size_t)((scratch_grid + kFinishGroup - 1) / kFinishGroup);
   const size_t round_vals = (size_t)kRoundBatchMax * 2 * (size_t)cfg->n_devices;
   HADFL_CUDA(h, cudaMalloc((void **)&h->d_round_partials, sizeof(double) * round_vals * (size_t)scratch_grid));
@@ -1554,7 +1568,7 @@ uint64_t hadfl_launch_count(const hadfl_handle *h) { return h ? h->launches : 0;
 int64_t hadfl_row_stride(const hadfl_handle *h) { return h ? h->stride : 0; }
 int32_t hadfl_round_grid(const hadfl_handle *h) {
   if (!h) return 0;
-  return rows_form(h, 1) ? (int32_t)rows_grid(h->cfg.n_devices, h->cfg.n_params) : h->round_grid;
+  return rows_form(h, 1) ? (int32_t)rows_grid(h->cfg.n_params, rows_groups(h->cfg.n_devices)) : h->round_grid;
 }
 
 int hadfl_selection_probs(const double *x, const uint8_t *avail, int32_t n, double *out_P) {

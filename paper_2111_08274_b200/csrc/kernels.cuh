@@ -1363,9 +1363,12 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
 // On large vectors the waits at the barrier, where all warps of a group are in the same phase, cost more
 // than registers save; there k_round is the faster one (the host decides: see rows_form).
 // A row moves to another warp from block to block, so that the heavy rows meet all SM sub-partitions.
-// Sums of a row: the fp32 part of the order is k_round's (a thread's pack, then the lanes l and l ^ 16), fp64 beyond.
+// Sums of a row: the fp32 part of the order is k_round's (a thread's pack, then the lanes l and l ^ 16), fp64 beyond;
+// the lanes' values wait in shared memory until the tile's rounds are done (a butterfly in each round stood between
+// two barriers: 8 rounds of 4 devices and 100,000 parameters 3.77 -> 3.73 us each).
 // ------------------------------------------------------------------------------------------
-constexpr int kRowsMaxThreads = 1024;
+// Threads of a block, at most: the build for 512 has twice the registers, for blocks that have an SM to themselves.
+constexpr int kRowsMaxThreads = 1024, kRowsFewThreads = 512;
 
 struct RowsStep {  // one device in one round
   int32_t steps;
@@ -1403,16 +1406,18 @@ struct SelectedRow {
   }
 };
 
-// Dynamic shared memory of a block: [group][2][k] selected rows, [group][round][n][2] row sums.
+// Dynamic shared memory of a block: [group][2][k] selected rows, [group][round][n][2] row sums, [warp][round][32]
+// what a row's lanes have to add in a tile.
+__host__ __device__ constexpr int rows_slots(int rounds) { return (rounds + 3) / 4 * 4; }  // four rounds are added at a time
 template <typename WT, int E>
 constexpr size_t rows_selected_bytes(int k) { return (size_t)2 * k * SelectedRow<WT, E>::kBytes; }
 template <typename WT, int E>
 constexpr size_t rows_shared_bytes(int groups, int n, int k, int rounds) {
-  return groups * (rows_selected_bytes<WT, E>(k) + sizeof(double) * 2 * n * rounds);
+  return groups * (rows_selected_bytes<WT, E>(k) + sizeof(double) * 2 * n * rounds + sizeof(float) * 32 * n * rows_slots(rounds));
 }
 
-template <typename WT, typename MT, typename Gen, int E, int RM, int NR>
-__global__ void __launch_bounds__(kRowsMaxThreads)
+template <typename WT, typename MT, typename Gen, int E, int RM, int NR, int kMaxThreads>
+__global__ void __launch_bounds__(kMaxThreads)
 k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_params,
              PhiloxKeys keys, StepConsts k, RoundScratch scratch, const __grid_constant__ RowsBatch<NR> b) {
   using Sel = SelectedRow<WT, E>;
@@ -1427,6 +1432,7 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
   char *sel = s_rows + group * 2 * n_sel * Sel::kBytes;
   double *all_sums = reinterpret_cast<double *>(s_rows + groups * 2 * n_sel * Sel::kBytes);
   double *sums = all_sums + group * n_vals + 2 * row;  // each owned by the warp of that row
+  float *slots = reinterpret_cast<float *>(all_sums + groups * n_vals) + warp * rows_slots(n_rounds) * 32;
   for (int t = threadIdx.x; t < groups * n_vals; t += blockDim.x) all_sums[t] = 0.0;
   RowStep rs;
   rs.row = row;
@@ -1439,7 +1445,9 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 
   const int64_t n_packs = (n_params + E - 1) / E;
   const int64_t n_tiles = (n_packs + 31) / 32;
-  for (int64_t tile = (int64_t)blockIdx.x * groups + group; tile < n_tiles; tile += (int64_t)gridDim.x * groups) {
+  // (warps beyond the groups' are there for the finish)
+  for (int64_t tile = group < groups ? (int64_t)blockIdx.x * groups + group : n_tiles; tile < n_tiles;
+       tile += (int64_t)gridDim.x * groups) {
     auto do_tile = [&](auto all_full) {
       const int64_t p = tile * 32 + lane;
       const auto live = live_of<E>(all_full, n_params, p);
@@ -1524,10 +1532,17 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
           d2 = fmaf(d, d, d2);
         }
         const bool upper = (lane & 16) != 0;
-        double d = (double)((upper ? d2 : n2) + __shfl_xor_sync(0xFFFFFFFFu, upper ? n2 : d2, 16));
-#pragma unroll
-        for (int off = 8; off > 0; off >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, off);
-        if ((lane & 15) == 0) sums[r * 2 * n + (lane >> 4)] += d;  // lower half-warp norms, upper distances
+        slots[r * 32 + lane] = (upper ? d2 : n2) + __shfl_xor_sync(0xFFFFFFFFu, upper ? n2 : d2, 16);
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int r0 = 0; r0 < n_rounds; r0 += 4) {  // 8 lanes per round: 4 add its norms, 4 its distances
+        const float4 v = reinterpret_cast<const float4 *>(slots + r0 * 32)[lane];
+        double d = ((double)v.x + (double)v.y) + ((double)v.z + (double)v.w);
+        d += __shfl_xor_sync(0xFFFFFFFFu, d, 1);
+        d += __shfl_xor_sync(0xFFFFFFFFu, d, 2);
+        const int r = r0 + (lane >> 3);
+        if ((lane & 3) == 0 && r < n_rounds) sums[r * 2 * n + ((lane >> 2) & 1)] += d;
       }
       if (w_changed) st_pack_any(wp, 0, live, wv);
       if (m_changed) st_pack_any(mp, 0, live, mv);

@@ -82,3 +82,12 @@ def test_reported_grid_is_that_of_a_single_round(n, P):
     columns = 256 * max(8 // n, 1) if rows else 2048
     assert a.h.round_grid() == -(-P // columns)
     a.close()
+
+
+@pytest.mark.parametrize("dtype,m_dtype,rounding", STORAGE)
+@pytest.mark.parametrize("n,per_sm,over", [(1, 8, 0), (1, 8, 1), (2, 8, 0), (2, 8, 1), (3, 5, 0), (3, 5, 1), (4, 1, 0), (4, 1, 1),
+                                           (4, 3, 1), (4, 4, 0), (16, 1, 0), (16, 1, 1)])
+def test_batches_with_an_sm_per_block(n, per_sm, over, dtype, m_dtype, rounding):
+    """Tiles on both sides of what blocks of 16 warps hold with one block on every SM."""
+    tiles = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + over
+    test_rows_form_against_the_separate_calls(n, 256 * tiles - 3, max(1, n // 3), dtype, m_dtype, rounding)
