@@ -945,12 +945,14 @@ __device__ __forceinline__ void finish_by_last_block(const double *__restrict__ 
 // group order and hands them to `emit`.  Each of the two sums has a fixed order that does not
 // depend on which block happens to compute it, so the result is reproducible; no block waits for
 // another; all tickets are back at zero when the launch ends.
-// Launches with few partial sums in all (values x blocks) are one group: a second level's fence, ticket and loads come
-// after the last block's work, and what that block then has to add takes less.  Measured, us per launch of one round,
-// two levels / one: 4 devices, 100,000 parameters (1,568 sums) 8.5 / 7.0; 16 devices, 65,536 (8,192) 12.2 / 10.6; 4
-// devices, 300,001 (4,696) 11.4 / 9.6; 8 devices, 1,000,000 (7,824) 31.6 / 31.1; two rounds of 4 devices, 100,000 11.5 / 10.0.
+// Launches of few blocks are one group: a second level's fence, ticket and loads come after the last block's work.  One
+// block then adds everything, its warps two values at a time (a turn) and 128 blocks' sums of each at a time, one wait
+// for L2 after the other: up to 2 x 128 blocks that costs less than the second level, up to 4 x 128 with two turns at
+// most, and beyond that it grows with the blocks.  Measured, us per launch of one round, two levels / one (values x
+// blocks): 4 devices 8 x 196 8.8 / 7.3, 8 x 512 13.5 / 12.9, 8 x 2048 49.8 / 55.0; 2 devices 4 x 4096 50.4 / 63.2; one
+// device 2 x 512 7.7 / 6.9, 2 x 1024 11.0 / 11.7, 2 x 8192 58.0 / 80.7; 16 devices 32 x 256 26.4 / 24.6; 32 devices 64 x
+// 256 59.2 / 56.4, 64 x 512 96.8 / 97.9; 8 devices 16 x 512 21.2 / 20.6, 16 x 1024 48.2 / 49.4.
 constexpr int kFinishGroup = 128;
-constexpr int kFinishFlat = 16384;
 
 template <typename Emit>
 __device__ __forceinline__ void finish_two_level(const double *__restrict__ partials,
@@ -959,11 +961,12 @@ __device__ __forceinline__ void finish_two_level(const double *__restrict__ part
                                                  unsigned int *__restrict__ ticket, bool *s_last,
                                                  Emit emit) {
   const int n_blocks = (int)gridDim.x;
-  const int group = n_vals * n_blocks <= kFinishFlat ? n_blocks : kFinishGroup;
-  const int n_groups = (n_blocks + group - 1) / group;
-  const int g = (int)blockIdx.x / group;
-  const int g_first = g * group;
-  const int g_size = min(group, n_blocks - g_first);
+  const int two_turns = (int)blockDim.x / 8;  // values: 2 x 2 per warp
+  const bool one_level = n_blocks <= 2 * kFinishGroup || (n_blocks <= 4 * kFinishGroup && n_vals <= two_turns);
+  const int n_groups = one_level ? 1 : (n_blocks + kFinishGroup - 1) / kFinishGroup;
+  const int g = one_level ? 0 : (int)blockIdx.x / kFinishGroup;
+  const int g_first = g * kFinishGroup;
+  const int g_size = one_level ? n_blocks : min(kFinishGroup, n_blocks - g_first);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) *s_last = (atomicAdd(group_tickets + g, 1u) == (unsigned)g_size - 1u);

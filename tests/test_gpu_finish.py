@@ -57,3 +57,18 @@ def test_one_group_and_several(blocks, rounds):
         sel = arena.run_rounds_fused(first, rounds)[-1]
         check(arena.h.stats_read(), sums(arena, int(sel[0])), ROUND)
     arena.close()
+
+
+@pytest.mark.parametrize("n,blocks,rounds", [(2, 512, 1), (2, 513, 1), (16, 512, 1), (17, 257, 1), (24, 256, 2), (24, 257, 2),
+                                             (24, 384, 2), (32, 512, 1), (32, 513, 1), (1, 1024, 1), (1, 1025, 1)])
+def test_one_level_and_two(n, blocks, rounds):
+    """Both sides of the lines between a finish by one block and one in two levels: 256 blocks, 512 blocks, and the number
+    of values in between; in two levels with a last group of 128 blocks, of fewer and of one."""
+    wl = Workload("fin", n, 2048 * blocks - 1, max(1, n // 4), 1, "fixed", tuple(1 + i % 2 for i in range(n)), grad_std=1e-2,
+                  seed=workloads.BASE_SEED + blocks)
+    arena = runtime.Arena(wl)
+    for first in (0, rounds):                            # the tickets are back at zero for the second launch
+        sel = arena.run_rounds_fused(first, rounds)[-1]
+        check(arena.h.stats_read(), sums(arena, int(sel[0])), ROUND)
+    arena.h.debug_check()
+    arena.close()
