@@ -938,31 +938,78 @@ __device__ __forceinline__ void finish_by_last_block(const double *__restrict__ 
   if (threadIdx.x == 0) *ticket = 0u;
 }
 
-// Two-level variant for grids of many blocks (the fused round).  Blocks are grouped in runs of
+// Finish for grids of many blocks (the fused round), in two levels.  Blocks are grouped in runs of
 // kFinishGroup consecutive block indices.  The block that draws a group's last ticket sums that
 // group's partials[t][first block of the group ...] in block order -> group_partials[t][group]
 // and draws the launch's ticket; the block that draws the last of those sums the group sums in
 // group order and hands them to `emit`.  Each of the two sums has a fixed order that does not
 // depend on which block happens to compute it, so the result is reproducible; no block waits for
 // another; all tickets are back at zero when the launch ends.
-// Launches of few blocks are one group: a second level's fence, ticket and loads come after the last block's work.  One
-// block then adds everything, its warps two values at a time (a turn) and 128 blocks' sums of each at a time, one wait
-// for L2 after the other: up to 2 x 128 blocks that costs less than the second level, up to 4 x 128 with two turns at
-// most, and beyond that it grows with the blocks.  Measured, us per launch of one round, two levels / one (values x
-// blocks): 4 devices 8 x 196 8.8 / 7.3, 8 x 512 13.5 / 12.9, 8 x 2048 49.8 / 55.0; 2 devices 4 x 4096 50.4 / 63.2; one
-// device 2 x 512 7.7 / 6.9, 2 x 1024 11.0 / 11.7, 2 x 8192 58.0 / 80.7; 16 devices 32 x 256 26.4 / 24.6; 32 devices 64 x
-// 256 59.2 / 56.4, 64 x 512 96.8 / 97.9; 8 devices 16 x 512 21.2 / 20.6, 16 x 1024 48.2 / 49.4.
 constexpr int kFinishGroup = 128;
 
+// Both levels by one block, for up to 4 groups, in the same order: the order must not depend on which of the two a
+// launch takes, since that follows from its number of rounds and a batch leaves the statistics that single rounds do.
+// A warp takes two values of two groups at a time, all 16 loads of a lane in flight.  The butterflies over the lanes are
+// folded into one: lanes 0 .. 15 go on with the first value and 16 .. 31 with the second, the odd eights with the
+// second group, and every sum is that of the whole butterfly (lane l has what lane l of it would have).  The group sums
+// G0 .. G3 then meet as in the second level: (G0 + G2) + (G1 + G3).
 template <typename Emit>
-__device__ __forceinline__ void finish_two_level(const double *__restrict__ partials,
+__device__ __forceinline__ void sum_up_to_four_groups(const double *__restrict__ partials, int n_vals, int n_blocks, Emit emit) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  const bool second = (lane & 16) != 0, odd = (lane & 8) != 0;
+#pragma unroll 1
+  for (int t0 = warp * 2; t0 < n_vals; t0 += n_warps * 2) {
+    double sum = 0.0;
+#pragma unroll 1
+    for (int first = 0; first < n_blocks; first += 2 * kFinishGroup) {
+      double v[2][2][4], p[2][2] = {};
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int l = first + g * kFinishGroup + 32 * q + lane;
+            v[i][g][q] = t0 + i < n_vals && l < n_blocks ? __ldcg(partials + (int64_t)(t0 + i) * n_blocks + l) : 0.0;
+          }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) p[i][g] += v[i][g][q];
+      double d[2];
+#pragma unroll
+      for (int g = 0; g < 2; ++g)
+        d[g] = (second ? p[1][g] : p[0][g]) + __shfl_xor_sync(0xFFFFFFFFu, second ? p[0][g] : p[1][g], 16);
+      double s = (odd ? d[1] : d[0]) + __shfl_xor_sync(0xFFFFFFFFu, odd ? d[0] : d[1], 8);
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+      sum += s;
+    }
+    sum += __shfl_xor_sync(0xFFFFFFFFu, sum, 8);
+    const int t = t0 + (lane >> 4);
+    if ((lane & 15) == 0 && t < n_vals) emit(t, sum);
+  }
+}
+
+// Launches of few blocks are finished by one block, the last one: a second level's fence, ticket and loads come after
+// the last block's work.  One block's warps add two values at a time (a turn) and two groups of each at a time, one wait
+// for L2 after the other: up to 2 groups that costs less than the second level, up to 4 with four turns at most, and
+// beyond that it grows with the blocks.  Measured, us per launch of one round, two levels / one (values x blocks): 4
+// devices 8 x 196 8.8 / 6.8, 8 x 512 13.5 / 12.2; one device 2 x 512 7.7 / 6.3; 16 devices 32 x 256 26.2 / 23.7; 32
+// devices 64 x 256 58.5 / 54.4, 64 x 512 97.1 / 95.9; 8 rounds in one launch, 512 x 147 53.2 / 48.7 per round.  Beyond the
+// lines (one level as one sequence of all the blocks' sums): one device 2 x 1024 11.1 / 11.7, 2 x 8192 57.6 / 80.1; 2 devices
+// 4 x 4096 50.1 / 62.7; 8 devices 16 x 1024 48.0 / 49.2.
+template <typename Emit>
+__device__ __forceinline__ void finish_by_groups(const double *__restrict__ partials,
                                                  double *__restrict__ group_partials, int n_vals,
                                                  unsigned int *__restrict__ group_tickets,
                                                  unsigned int *__restrict__ ticket, bool *s_last,
                                                  Emit emit) {
   const int n_blocks = (int)gridDim.x;
-  const int two_turns = (int)blockDim.x / 8;  // values: 2 x 2 per warp
-  const bool one_level = n_blocks <= 2 * kFinishGroup || (n_blocks <= 4 * kFinishGroup && n_vals <= two_turns);
+  const int four_turns = (int)blockDim.x / 4;  // values: 4 x 2 per warp
+  const bool one_level = n_blocks <= 2 * kFinishGroup || (n_blocks <= 4 * kFinishGroup && n_vals <= four_turns);
   const int n_groups = one_level ? 1 : (n_blocks + kFinishGroup - 1) / kFinishGroup;
   const int g = one_level ? 0 : (int)blockIdx.x / kFinishGroup;
   const int g_first = g * kFinishGroup;
@@ -973,17 +1020,14 @@ __device__ __forceinline__ void finish_two_level(const double *__restrict__ part
   __syncthreads();
   if (!*s_last) return;
   __threadfence();
-  sum_partials(partials + g_first, n_blocks, n_vals, g_size, [&](int t, double s) {
-    if (n_groups == 1) {  // a single group: its sum is the result (the second level would add 0 to it)
-      emit(t, s);
-    } else if (access_ok(group_partials + (int64_t)t * n_groups + g, 8)) {
-      group_partials[(int64_t)t * n_groups + g] = s;
-    }
-  });
-  if (n_groups == 1) {
-    if (threadIdx.x == 0) group_tickets[g] = 0u;
+  if (one_level) {
+    sum_up_to_four_groups(partials, n_vals, n_blocks, emit);
+    if (threadIdx.x == 0) group_tickets[0] = 0u;
     return;
   }
+  sum_partials(partials + g_first, n_blocks, n_vals, g_size, [&](int t, double s) {
+    if (access_ok(group_partials + (int64_t)t * n_groups + g, 8)) group_partials[(int64_t)t * n_groups + g] = s;
+  });
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1110,7 +1154,7 @@ k_stats(const WT *__restrict__ w, int64_t stride, int64_t n_params, int n_device
 // Row sums: one shuffle per row and pack, then a shared-memory slot owned by the thread (fp32); at
 // the end of a chunk's round, per row, a fixed-order sum over the warps and a butterfly over each
 // half-warp (fp64), added to the block's sums of that round; at the end of the block
-// partials[round][value][block] and one two-level last-ticket finish.  Deterministic.
+// partials[round][value][block] and one last-ticket finish.  Deterministic.
 // Dynamic shared memory: n * kThreads floats.  64 registers: four resident blocks per SM.
 // NR > 1: the launch takes a batch of up to NR consecutive rounds.  A block carries its chunk
 // through all of them before it moves on (chunk loop outside, round loop inside), so from the
@@ -1331,7 +1375,7 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
     else
       do_chunk(std::false_type{});
   }
-  // ---- launch: partials[round][value][block], then one two-level last-ticket finish for all rounds (one
+  // ---- launch: partials[round][value][block], then one last-ticket finish for all rounds (one
   // fence and one ticket per block)
   const int n_rounds = NR == 1 ? 1 : b.n_rounds;
   const int n_vals = n_rounds * 2 * n_dev;
@@ -1340,7 +1384,7 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
     double *slot = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
     if (access_ok(slot, 8)) *slot = s_part[r][t - r * 2 * n_dev];
   }
-  finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
+  finish_by_groups(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
                    [&](int t, double sum) {
     const int r = NR == 1 ? 0 : t / (2 * n_dev), v = t - r * 2 * n_dev, j = v >> 1, which = v & 1;
     const RoundArgs &a = b.round[r];
@@ -1564,8 +1608,8 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
     double *at = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
     if (access_ok(at, 8)) *at = d;
   }
-  // one two-level finish over all rounds of the batch (one fence and one ticket per block)
-  finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
+  // one finish over all rounds of the batch (one fence and one ticket per block)
+  finish_by_groups(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
                    [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, at = (v & 1) * n + (v >> 1);  // [norms of the rows][distances]
     const bool holder = b.s[r][v >> 1].visit < n_sel;  // of the aggregate: at distance 0, whatever its values
@@ -2044,7 +2088,7 @@ k_rounds_resident(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, Phil
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(cols));
 
-  finish_two_level(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
+  finish_by_groups(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
                    [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, j = v >> 1, which = v & 1;
     auto put = [&](int at, float x) { scratch.put(r, b.n_rounds, at, x); };

@@ -1,0 +1,46 @@
+"""The order of the statistics' sums is that of a launch of one round in a batch of any length of the same form of the
+kernel: the results are the same bit for bit, also where the order decides them.
+
+A row's squares are 2^53 + 2^29, halfway between two neighbours in fp32, in its first tile, and ones far apart.  In 64
+bits a one is lost beside the large sum and two of them are not, so the row's norm in fp32 shows whether ones met
+before they came to it."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_common import require_gpu
+from paper_2111_08274_b200 import runtime, workloads
+from paper_2111_08274_b200.workloads import Workload
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def check_order(n, P, ones, rounds):
+    wl = Workload("order", n, P, 1, 1, "fixed", (0,) * n, seed=workloads.BASE_SEED + P)
+    a = runtime.Arena(wl)
+    a.w.zero_()
+    a.w[:, 0:32:8] = torch.tensor([2.0 ** 26, 2.0 ** 26, 2.0 ** 14, 2.0 ** 14], device=a.device)
+    for c in ones:
+        a.w[:, c] = 1.0
+    torch.cuda.synchronize()
+    a.run_round_fused(0)
+    single, _ = a.h.stats_read()
+    assert np.isin(single, [2.0 ** 53, 2.0 ** 53 + 2.0 ** 30]).all()
+    for several in rounds:
+        a.run_rounds_fused(1, several)
+        for back in range(several):
+            assert np.array_equal(a.h.stats_read_round(back)[0], single), (several, back)
+    a.h.debug_check()
+    a.close()
+
+
+@pytest.mark.parametrize("blocks", [(32, 64), (128, 160), (33, 129), (256, 128), (256, 288), (1, 300)])
+def test_row_walk(blocks):
+    """24 devices, 2 groups of blocks and a bit, 3, and 4: one round is finished in one level, several in two."""
+    for n_blocks in (257, 301, 384, 512):
+        check_order(24, 2048 * n_blocks - 3, [2048 * b + 8 * i for i, b in enumerate(blocks) if b < n_blocks], (2, 3))
