@@ -31,7 +31,7 @@ struct hadfl_handle {
   int l2_bytes = 0;
   size_t smem_per_sm = 0;
   int smem_per_block = 0;                   // most shared memory of a block, static and dynamic
-  bool rows_smem[3] = {};                   // allow_all_shared is done for k_round_rows (one round, batches, batches of a block per SM)
+  bool rows_smem[2][2] = {};                // allow_all_shared is done for k_round_rows [up to 512 threads][batches]
   bool resident_smem[3] = {};               // ... for the builds of k_rounds_resident
   size_t resident_arena_bytes = 0;  // batches on arenas beyond this are resident on the SMs
   PhiloxKeys keys;
@@ -400,9 +400,31 @@ int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
 // all 16 warps, for the finish.  Measured, us per round of a batch of 8, tiles for 8 warps / one block per SM / the same
 // without the warps for the finish: 4 devices, 100,000 parameters 3.54 / 2.83 / 2.95, 30,000 2.72 / 2.10 / 2.65; 2 devices,
 // 300,001 2.53 / 2.12 / 2.12, 30,000 1.78 / 1.42 / 2.07; 8 devices, 70,001 4.88 / 4.25; 16 devices, 37,000 5.38 / 5.17.
+// (1 and 2 devices: 4 tiles instead of 3, see rows_units.)
 int rows_groups_one_per_sm(const hadfl_handle *h) {
-  const int64_t most = kRowsFewThreads / 32 / h->cfg.n_devices, tiles = rows_tiles(h->cfg.n_params);
-  return tiles <= h->sm_count * (most < 8 ? most : 8) ? (int)((tiles + h->sm_count - 1) / h->sm_count) : 0;
+  const int n = h->cfg.n_devices;
+  const int64_t most = kRowsFewThreads / 32 / n, tiles = rows_tiles(h->cfg.n_params);
+  if (tiles > h->sm_count * (most < 8 ? most : 8) || h->sm_count < 128 || h->sm_count > kPartSums) return 0;
+  const int groups = (int)((tiles + h->sm_count - 1) / h->sm_count);
+  return groups == 3 && n <= 2 ? 4 : groups;
+}
+// The statistics of single rounds are those of a batch bit for bit, so both add the tiles' sums in one order: that of the
+// blocks of the batch, since it has more of them to add.  A block first adds as many tiles at a time (a unit) as both kinds
+// of blocks are made of; those sums a block of the batch adds to one.  Blocks of a single round leave them as they are,
+// and the last one adds what belongs together: 1 to 3 of them (single rounds have up to 512 tiles; 128 to 160 SMs).
+// Measured, us per single round, sums of its own blocks in a build with half the registers / so, with the batch's
+// registers: 4 devices, 100,000 parameters 6.8 / 6.9, 70,001 6.2 / 5.9; 2 devices, 100,000 5.1 / 4.8; 5 devices, 70,001 6.9 /
+// 6.5; 8 devices, 70,001 7.8 / 7.4.  Batches with their tiles' sums apart instead, for the order of single rounds: 2.82 /
+// 3.05 per round (4 devices, 100,000), 2.62 / 2.90 (5 devices, 70,001).
+RowsUnits rows_units(const hadfl_handle *h, int groups, int groups_single) {
+  RowsUnits u;
+  u.tiles = groups < groups_single ? groups : groups_single;
+  while (groups % u.tiles || groups_single % u.tiles) --u.tiles;
+  u.parts = groups / u.tiles;
+  u.per_block = groups_single / u.tiles;
+  u.n_units = (int)((rows_tiles(h->cfg.n_params) + u.tiles - 1) / u.tiles);
+  u.n_sums = (u.n_units + u.parts - 1) / u.parts;
+  return u;
 }
 
 template <int NR>
@@ -415,8 +437,9 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
     q.n = h->cfg.n_devices;
     q.k = b.round[0].k;
     q.n_rounds = b.n_rounds;
-    const int few = NR > 1 ? rows_groups_one_per_sm(h) : 0;
-    q.groups = few ? few : rows_groups(q.n);
+    const int few = rows_groups_one_per_sm(h);
+    q.groups = NR > 1 && few ? few : rows_groups(q.n);
+    if (few) q.units = rows_units(h, few, rows_groups(q.n));
     q.beta = b.round[0].beta;
     q.one_minus_beta = b.round[0].one_minus_beta;
     for (int r = 0; r < b.n_rounds; ++r) {
@@ -428,11 +451,10 @@ int launch_round_rows(hadfl_handle *h, const RoundBatch<NR> &b, float lr, const 
     const int grid = (int)rows_grid(h->cfg.n_params, q.groups);
     const size_t smem = rows_shared_bytes<WT, E>(q.groups, q.n, q.k, b.n_rounds);
     auto kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR, kRowsMaxThreads>;
-    if constexpr (NR > 1)
-      if (few) kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR, kRowsFewThreads>;
-    const int rc = allow_all_shared(h, kernel, h->rows_smem[few ? 2 : NR > 1]);
+    if (few) kernel = k_round_rows<WT, MT, NormalsFast, E, decltype(rm)::value, NR, kRowsFewThreads>;
+    const int rc = allow_all_shared(h, kernel, h->rows_smem[few != 0][NR > 1]);
     if (rc != HADFL_OK) return rc;
-    const int threads = few ? kRowsFewThreads : q.groups * q.n * 32;
+    const int threads = NR > 1 && few ? kRowsFewThreads : q.groups * q.n * 32;
     kernel<<<grid, threads, smem, h->stream>>>((WT *)h->w, (MT *)h->m, h->stride, h->cfg.n_params, h->keys,
                                                step_consts(h, lr), scratch, q);
     h->last_launch_pack = E;

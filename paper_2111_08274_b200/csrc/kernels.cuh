@@ -920,6 +920,17 @@ __device__ __forceinline__ void sum_partials(const double *__restrict__ src, int
   }
 }
 
+// Whether this block draws the last of n tickets; what it wrote before is visible to the block that does.
+__device__ __forceinline__ bool is_last_block(unsigned int *__restrict__ ticket, unsigned int n, bool *s_last) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) *s_last = (atomicAdd(ticket, 1u) == n - 1u);
+  __syncthreads();
+  if (!*s_last) return false;
+  __threadfence();
+  return true;
+}
+
 // Last-block finish: the block that draws the last ticket sums partials[t][0 .. n_src) for every
 // t < n_vals in a fixed order (a warp per value, lanes strided, then the butterfly), hands the
 // sums to `emit`, and resets the ticket.  Returns without waiting for anyone.
@@ -928,12 +939,7 @@ __device__ __forceinline__ void finish_by_last_block(const double *__restrict__ 
                                                      int n_vals, int n_src,
                                                      unsigned int *__restrict__ ticket,
                                                      bool *s_last, Emit emit) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) *s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
+  if (!is_last_block(ticket, gridDim.x, s_last)) return;
   sum_partials(partials, n_src, n_vals, n_src, emit);
   if (threadIdx.x == 0) *ticket = 0u;
 }
@@ -993,6 +999,44 @@ __device__ __forceinline__ void sum_up_to_four_groups(const double *__restrict__
   }
 }
 
+// The same for up to kPartSums sums that are in kParts parts each, which are added first: part i of sum s is number
+// s * kParts + i of the n_src, and at partials[value][i][s].  All loads of a lane in flight, without a condition (one that
+// waits for the load before it costs as much again); what lies beyond the end is left out afterwards.
+constexpr int kPartSums = 160;
+template <int kParts, typename Emit>
+__device__ __forceinline__ void sum_parts(const double *__restrict__ partials, int n_vals, int n_src, int n_sums, Emit emit) {
+  constexpr int kVals = kParts == 2 ? 2 : 1, kLoads = kPartSums / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  const bool upper = (lane & 16) != 0;
+#pragma unroll 1
+  for (int t0 = warp * kVals; t0 < n_vals; t0 += n_warps * kVals) {
+    const double *mine = partials + t0 * kParts * n_sums;
+    double v[kVals][kParts][kLoads];
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const double *at = mine + min(32 * q + lane, n_sums - 1);
+#pragma unroll
+      for (int i = 0; i < kVals * kParts; ++i, at += n_sums) v[i / kParts][i % kParts][q] = __ldcg(at);
+    }
+#pragma unroll
+    for (int k = 0; k < kVals; ++k) {
+      double p[2] = {};
+#pragma unroll
+      for (int q = 0; q < kLoads; ++q) {
+        double sum = 0.0;
+#pragma unroll
+        for (int i = 0; i < kParts; ++i) sum += (32 * q + lane) * kParts + i < n_src ? v[k][i][q] : 0.0;
+        p[32 * q / kFinishGroup] += sum;
+      }
+      double s = (upper ? p[1] : p[0]) + __shfl_xor_sync(0xFFFFFFFFu, upper ? p[0] : p[1], 16);
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+      s += __shfl_xor_sync(0xFFFFFFFFu, s, 16);
+      if (lane == 0) emit(t0 + k, s);
+    }
+  }
+}
+
 // Launches of few blocks are finished by one block, the last one: a second level's fence, ticket and loads come after
 // the last block's work.  One block's warps add two values at a time (a turn) and two groups of each at a time, one wait
 // for L2 after the other: up to 2 groups that costs less than the second level, up to 4 with four turns at most, and
@@ -1014,12 +1058,7 @@ __device__ __forceinline__ void finish_by_groups(const double *__restrict__ part
   const int g = one_level ? 0 : (int)blockIdx.x / kFinishGroup;
   const int g_first = g * kFinishGroup;
   const int g_size = one_level ? n_blocks : min(kFinishGroup, n_blocks - g_first);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) *s_last = (atomicAdd(group_tickets + g, 1u) == (unsigned)g_size - 1u);
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
+  if (!is_last_block(group_tickets + g, (unsigned)g_size, s_last)) return;
   if (one_level) {
     sum_up_to_four_groups(partials, n_vals, n_blocks, emit);
     if (threadIdx.x == 0) group_tickets[0] = 0u;
@@ -1028,15 +1067,8 @@ __device__ __forceinline__ void finish_by_groups(const double *__restrict__ part
   sum_partials(partials + g_first, n_blocks, n_vals, g_size, [&](int t, double s) {
     if (access_ok(group_partials + (int64_t)t * n_groups + g, 8)) group_partials[(int64_t)t * n_groups + g] = s;
   });
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    group_tickets[g] = 0u;
-    *s_last = (atomicAdd(ticket, 1u) == (unsigned)n_groups - 1u);
-  }
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
+  if (threadIdx.x == 0) group_tickets[g] = 0u;
+  if (!is_last_block(ticket, (unsigned)n_groups, s_last)) return;
   sum_partials(group_partials, n_groups, n_vals, n_groups, emit);
   if (threadIdx.x == 0) *ticket = 0u;
 }
@@ -1414,7 +1446,8 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
 // the lanes' values wait in shared memory until the tile's rounds are done (a butterfly in each round stood between
 // two barriers: 8 rounds of 4 devices and 100,000 parameters 3.77 -> 3.73 us each).
 // ------------------------------------------------------------------------------------------
-// Threads of a block, at most: the build for 512 has twice the registers, for blocks that have an SM to themselves.
+// Threads of a block, at most: the build for 512 has twice the registers, for batches whose blocks have an SM to
+// themselves and for single rounds of the same vectors.
 constexpr int kRowsMaxThreads = 1024, kRowsFewThreads = 512;
 
 struct RowsStep {  // one device in one round
@@ -1422,10 +1455,17 @@ struct RowsStep {  // one device in one round
   uint32_t base_lo, r1_c2;  // as in RowStep
   int32_t visit;            // position in the draw (0 .. k - 1: selected), or k and above
 };
+struct RowsUnits {  // the order of the tiles' sums
+  int32_t tiles;             // are added first, to a unit's
+  int32_t parts;             // units of a block of a batch
+  int32_t per_block;         // units of a block of a single round
+  int32_t n_units, n_sums;   // units of the vector, and blocks of a batch
+};
 template <int NR>
 struct RowsBatch {
   int32_t n, k, n_rounds;
   int32_t groups;             // tiles that a block has in hand at a time
+  RowsUnits units;            // (blocks of up to kRowsFewThreads)
   float beta, one_minus_beta;
   int32_t write_all[NR];      // as in RoundArgs
   float a[NR][kMaxDevices];   // aggregation weights in draw order
@@ -1602,19 +1642,49 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
       do_tile(std::false_type{});
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < n_vals; t += blockDim.x) {
-    double d = 0.0;
-    for (int g = 0; g < groups; ++g) d += all_sums[g * n_vals + t];
-    double *at = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
-    if (access_ok(at, 8)) *at = d;
-  }
-  // one finish over all rounds of the batch (one fence and one ticket per block)
-  finish_by_groups(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last,
-                   [&](int t, double sum) {
+  auto put = [&](int t, double sum) {
     const int r = t / (2 * n), v = t - r * 2 * n, at = (v & 1) * n + (v >> 1);  // [norms of the rows][distances]
     const bool holder = b.s[r][v >> 1].visit < n_sel;  // of the aggregate: at distance 0, whatever its values
     scratch.put(r, n_rounds, at, holder && (v & 1) ? 0.f : (float)sum);
-  });
+  };
+  if constexpr (kMaxThreads == kRowsFewThreads && NR == 1) {
+    // the sums of a batch's blocks, which are not this launch's (see rows_units): the warps of a tile's rows store them
+    const auto &u = b.units;
+    const int at_unit = (int)blockIdx.x * u.per_block + group;
+    if (group < u.per_block && at_unit < u.n_units && lane < 2) {
+      const int t = 2 * (warp - group * n) + lane;
+      const int sum = u.parts == 1 ? at_unit : u.parts == 2 ? at_unit / 2 : at_unit / 3;
+      double d = 0.0;
+      for (int g = group * u.tiles; g < (group + 1) * u.tiles; ++g) d += all_sums[g * n_vals + t];
+      double *at = scratch.partials + (t * u.parts + at_unit - sum * u.parts) * u.n_sums + sum;
+      if (access_ok(at, 8)) *at = d;
+    }
+    if (!is_last_block(scratch.tickets, gridDim.x, &s_last)) return;
+    if (u.parts == 1)
+      sum_up_to_four_groups(scratch.partials, n_vals, u.n_sums, put);
+    else if (u.parts == 2)
+      sum_parts<2>(scratch.partials, n_vals, u.n_units, u.n_sums, put);
+    else
+      sum_parts<3>(scratch.partials, n_vals, u.n_units, u.n_sums, put);
+    if (threadIdx.x == 0) scratch.tickets[0] = 0u;
+  } else {
+    for (int t = threadIdx.x; t < n_vals; t += blockDim.x) {
+      double d = 0.0;
+      if (kMaxThreads == kRowsFewThreads) {
+        for (int g0 = 0; g0 < groups; g0 += b.units.tiles) {
+          double of_unit = 0.0;
+          for (int g = g0; g < g0 + b.units.tiles; ++g) of_unit += all_sums[g * n_vals + t];
+          d += of_unit;
+        }
+      } else {
+        for (int g = 0; g < groups; ++g) d += all_sums[g * n_vals + t];
+      }
+      double *at = scratch.partials + (int64_t)t * gridDim.x + blockIdx.x;
+      if (access_ok(at, 8)) *at = d;
+    }
+    // one finish over all rounds of the batch (one fence and one ticket per block)
+    finish_by_groups(scratch.partials, scratch.group_partials, n_vals, scratch.tickets + 1, scratch.tickets, &s_last, put);
+  }
 }
 
 // ------------------------------------------------------------------------------------------

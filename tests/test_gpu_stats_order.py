@@ -44,3 +44,13 @@ def test_row_walk(blocks):
     """24 devices, 2 groups of blocks and a bit, 3, and 4: one round is finished in one level, several in two."""
     for n_blocks in (257, 301, 384, 512):
         check_order(24, 2048 * n_blocks - 3, [2048 * b + 8 * i for i, b in enumerate(blocks) if b < n_blocks], (2, 3))
+
+
+@pytest.mark.parametrize("tiles", [(64, 256), (1, 2), (2, 3), (3, 4), (5, 131), (63, 65), (128, 130), (37, 101)])
+@pytest.mark.parametrize("n,P", [(1, 37_889), (1, 131_072), (2, 30_001), (2, 100_001), (2, 131_071), (3, 37_888), (3, 113_663), (4, 30_000),
+                                 (4, 37_889), (4, 100_000), (4, 131_072), (5, 113_664), (5, 113_665), (7, 70_001), (8, 37_889), (8, 75_776),
+                                 (8, 75_777), (16, 37_888)])
+def test_warp_per_row(n, P, tiles):
+    """One to four tiles per block in a batch, where one round has eight, four, two or one: the most that an SM takes in
+    one block, one tile more, and in between."""
+    check_order(n, P, [min(256 * t + 8, P - 1) for t in tiles], (2, 5, 8))
