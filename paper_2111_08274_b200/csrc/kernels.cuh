@@ -508,7 +508,14 @@ __device__ __forceinline__ void sgd_update_pair(float &w0, float &w1, float &m0,
 // warp instructions out of a step of an 8-parameter pack (measured: K1 -3 ... -4 %, fused round
 // -4 ... -5 %).
 // The gradient noise of step e for the NB column groups of a pack: nz[b] = grad_std * (z0, z1), (z2, z3).
-template <typename Gen, int NB>
+// kVote: whether the rare logarithm series (about once in 250 steps of a pack) is asked for by the warp, so that the
+// branch is taken by all lanes or by none and needs no convergence point; all lanes of the warp run the step then.
+// Measured, us, lane / warp: ResNet-18 size, 8 steps per device, fp32 local update 557.1 / 555.4, fused round 575.9 /
+// 574.0; bf16 throughout, stochastic rounding, steps 1,1,2,2,4,4,8,8 2240 / 2236; batches of 16 devices with those
+// steps 807.5 / 805.9; 32 devices, 2 M, bf16 parameters, one step 172 / 173.  Two builds for bf16 parameters with fp32
+// momentum lose by it and ask each lane: the local update (8 steps 565 / 582, 2 steps 197 / 200.5), and the batch with a
+// prefetch (32 devices, 2 M, 3 rounds 159 / 167; 16 devices, 1.5 M, 8 rounds 50.8 / 52.0), which spills more.
+template <typename Gen, int NB, bool kVote = true>
 __device__ __forceinline__ void step_noise(float2 (&nz)[NB][2], int e, const uint32_t (&c2_first)[NB],
                                            const GroupProducts<NB> &gp, const RowStep &rs, const PhiloxKeys &keys,
                                            const StepConsts &k) {
@@ -529,16 +536,15 @@ __device__ __forceinline__ void step_noise(float2 (&nz)[NB][2], int e, const uin
     r2[b] = Gen::radius2_pair(x[b][0], x[b][2], k.lg_scale);
     top = max(top, max(x[b][0], x[b][2]));
   }
-  // About once in 250 steps of a pack; asked for the warp, so that the branch is taken by all lanes or by none and
-  // needs no convergence point (8 steps per device, ResNet-18 size: fused round 577.6 -> 575.1 us, local update 557.7
-  // -> 555.8; batches of 16 devices, steps 1,1,2,2,4,4,8,8: 809.5 -> 806.5).  All lanes of the warp run the step.
-  if (__any_sync(0xFFFFFFFFu, Gen::needs_series(top))) {
+  bool series = Gen::needs_series(top);
+  if (kVote) series = __any_sync(0xFFFFFFFFu, series);
+  if (series) {
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       if (Gen::needs_series(x[b][0])) r2[b].x = r2_next_to_one(x[b][0], k.scale2);
       if (Gen::needs_series(x[b][2])) r2[b].y = r2_next_to_one(x[b][2], k.scale2);
     }
-    __syncwarp();
+    if (kVote) __syncwarp();
   }
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
@@ -563,7 +569,7 @@ __device__ __forceinline__ void step_update(float (&w)[4 * NB], float (&m)[4 * N
 // All steps of a row.  The loop is not unrolled: the copies
 // would compute the step-independent products of the generator more than once (fused round 584 -> 578
 // us at 8 steps per device, ResNet-18 size).
-template <typename Gen, int NB>
+template <typename Gen, int NB, bool kVote = true>
 __device__ __forceinline__ void sgd_steps(float (&w)[4 * NB], float (&m)[4 * NB],
                                           const GroupProducts<NB> &gp, const RowStep &rs,
                                           const PhiloxKeys &keys, const StepConsts &k) {
@@ -573,7 +579,7 @@ __device__ __forceinline__ void sgd_steps(float (&w)[4 * NB], float (&m)[4 * NB]
 #pragma unroll 1
   for (int e = 0; e < rs.steps; ++e) {
     float2 nz[NB][2];
-    step_noise<Gen, NB>(nz, e, c2_first, gp, rs, keys, k);
+    step_noise<Gen, NB, kVote>(nz, e, c2_first, gp, rs, keys, k);
     step_update<NB>(w, m, nz, k);
   }
 }
@@ -665,6 +671,7 @@ template <typename WT, typename MT, typename Gen, int E, int RM>
 __global__ void __launch_bounds__(kThreads)
 k_local_step(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, LocalStepArgs a,
              PhiloxKeys keys, StepConsts k) {
+  constexpr bool kVote = !(sizeof(WT) == 2 && sizeof(MT) == 4 && RM == 0);  // (measured at step_noise)
   const int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   // The body is compiled twice: for blocks whose packs are all full (`live` is then the constant
   // E and every ragged-tail test in the loads and stores folds away: 2-3 % fewer instructions per
@@ -681,7 +688,7 @@ k_local_step(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, LocalStep
       ld_raw(at_row<MT>(mp, a.r[j].m_off), live, rm);
     };
     auto body = [&](int j, float (&wv)[E], float (&mv)[E]) {
-      sgd_steps<Gen, E / 4>(wv, mv, gp, a.r[j], keys, k);
+      sgd_steps<Gen, E / 4, kVote>(wv, mv, gp, a.r[j], keys, k);
       if constexpr (RM == 1) round_stochastic<MT, false>(wv, mv, gp, a.r[j], keys);
       st_pack_any(at_row<WT>(wp, a.r[j].w_off), 0, live, wv);
       st_pack_any(at_row<MT>(mp, a.r[j].m_off), 0, live, mv);
@@ -1263,6 +1270,7 @@ template <typename WT, typename MT, typename Gen, int E, int RM, bool PF, int NR
 __global__ void __launch_bounds__(kThreads, PF ? kRoundBlocksPerSM - 1 : kRoundBlocksPerSM)
 k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR> b, PhiloxKeys keys,
         StepConsts k, RoundScratch scratch) {
+  constexpr bool kVote = !(sizeof(WT) == 2 && sizeof(MT) == 4 && RM == 0 && PF && NR > 1);  // (measured at step_noise)
   constexpr int kWarps = kThreads / 32;
   extern __shared__ float s_acc[];  // [n][kThreads]: per-thread row sums of the round in hand
   __shared__ double s_part[NR][2 * kMaxDevices];  // the block's sums, per round
@@ -1315,7 +1323,7 @@ k_round(WT *__restrict__ w, MT *__restrict__ m, int64_t n_params, RoundBatch<NR>
             float mv[E];
             unpack(rw, wv);
             unpack(rm, mv);
-            sgd_steps<Gen, E / 4>(wv, mv, gp, a.r[j], keys, k);
+            sgd_steps<Gen, E / 4, kVote>(wv, mv, gp, a.r[j], keys, k);
             if constexpr (RM == 1) round_stochastic<MT, false>(wv, mv, gp, a.r[j], keys);
             st_pack_any(at_row<MT>(mp, a.r[j].m_off), 0, live, mv);
             if constexpr (RM == 0) {
