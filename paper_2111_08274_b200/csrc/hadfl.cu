@@ -544,8 +544,8 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
       q.n_stepping[r] = n_stepping;
       q.first_store[r] = a.k == 1 && a.r[0].steps == 0;  // it ran no steps, and a_0 = 1
     }
-    const int64_t mean_steps_x2 = 2 * sum_steps / ((int64_t)n * b.n_rounds);
-    // Blocks per SM.  With more than two steps per device on average the launch is bound by arithmetic, and 6
+    const int64_t device_rounds = (int64_t)n * b.n_rounds;
+    // Blocks per SM.  With 2.5 and more steps per device on average the launch is bound by arithmetic, and 6
     // blocks are the fastest whatever they leave to the L2.  Otherwise the most, up to 5 (6, where those find
     // room for as many rows), whose rows in the arena stay within 55 % of the L2: 72 MB of them, with 16
     // devices and 6 blocks, already came back from HBM (478 against 431 us per round).
@@ -562,12 +562,17 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
       return (double)(n - rows_on_chip(blocks)) * blocks * h->sm_count * kResidentThreads * 8.0 * (sizeof(WT) + sizeof(MT));
     };
     int blocks_per_sm = kResidentMaxBlocks;
-    if (mean_steps_x2 <= 4) {
+    if (2 * sum_steps < 5 * device_rounds) {
       if (rows_on_chip(blocks_per_sm) < rows_on_chip(blocks_per_sm - 1)) --blocks_per_sm;
       while (blocks_per_sm > 2 && in_l2(blocks_per_sm) > 0.55 * h->l2_bytes) --blocks_per_sm;
     }
-    // one visit per row and round: fp32, up to 1.5 steps per device on average (measured at Resident::kPartOneVisit)
-    const bool one_visit = sizeof(WT) == 4 && rows_on_chip(blocks_per_sm) < n && mean_steps_x2 <= 3;
+    // One visit per row and round: fp32, where enough rows live in L2 (13 devices and more, of which 8 or 9 are on the SM)
+    // fewer than two steps per device on average, with 10 to 12 devices up to 1.25.  Measured, visits apart over one visit,
+    // 4.2 M and 16.8 M parameters, 2 to 8 rounds, at 1 / 1.5 / 1.75 steps: 9 devices 0.99 .. 1.02 / 0.99 .. 1.01 / 0.99 ..
+    // 1.005; 10 1.00 .. 1.01 / 0.99 .. 1.01 / 0.99 .. 1.01; 12 1.02 .. 1.03 / 1.00 .. 1.01 / 0.99 .. 1.00; 13 1.02 .. 1.03 /
+    // 1.01 .. 1.02 / 1.00 .. 1.01; 16 1.03 .. 1.04 / 1.01 .. 1.02 / 1.00 .. 1.01; two steps 1.005 (and see Resident).
+    const bool one_visit = sizeof(WT) == 4 && rows_on_chip(blocks_per_sm) < n &&
+                           (n > 12 ? sum_steps < 2 * device_rounds : n > 9 && 4 * sum_steps <= 5 * device_rounds);
     const int max_blocks = one_visit ? kResidentOneVisitMaxBlocks : kResidentMaxBlocks;
     if (blocks_per_sm > max_blocks) blocks_per_sm = max_blocks;
     q.n_on_chip = rows_on_chip(blocks_per_sm);

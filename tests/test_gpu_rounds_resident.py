@@ -122,6 +122,14 @@ def test_rounds_that_do_not_gain_are_launched_apart(n, storage, per_round, launc
 @pytest.mark.parametrize("n,k,steps,beta", [(16, 1, (0, 1), 1.0), (16, 1, (0, 1), 0.5), (16, 16, (1,), 1.0), (19, 2, (2, 0), 0.25),
                                             (32, 3, (1,), 1.0)])
 def test_one_visit_per_row(n, k, steps, beta):
-    """fp32, a part of the rows on the SM, up to 1.5 steps per device: a single selected device without steps,
+    """fp32, a part of the rows on the SM, fewer than two steps per device: a single selected device without steps,
     all selected, several steps beside none, overwritten and mixed rounds."""
     compare(n, 150_000_001 // (n * 8) + 3, k, tuple(steps[i % len(steps)] for i in range(n)), "fp32", beta, (8, 5), 2)
+
+
+@pytest.mark.parametrize("n", [9, 10, 12, 13, 16])
+@pytest.mark.parametrize("steps", [(1,), (1, 1, 1, 2), (1, 2), (1, 2, 2, 2), (2,)])
+def test_one_visit_or_visits_apart(n, steps):
+    """Both sides of the lines between one visit per row and visits apart: 9, 10 to 12, and 13 devices; 1.25 and 2 steps per
+    device; in two rounds, where six blocks share an SM, and in three."""
+    compare(n, 150_000_001 // (n * 8) + 3, 2, tuple(steps[i % len(steps)] for i in range(n)), "fp32", 0.5, (2, 3), 2)
