@@ -576,7 +576,8 @@ int launch_rounds_resident(hadfl_handle *h, const RoundBatch<kRoundBatchMax> &b,
     const int max_blocks = one_visit ? kResidentOneVisitMaxBlocks : kResidentMaxBlocks;
     if (blocks_per_sm > max_blocks) blocks_per_sm = max_blocks;
     q.n_on_chip = rows_on_chip(blocks_per_sm);
-    // As much shared memory as keeps the number of blocks at that.
+    // As much shared memory as keeps the number of blocks at that (at the most that a build is planned with it may be
+    // one more, see kResidentOneVisitMaxBlocks).
     size_t smem = q.n_on_chip * kRowBytes + sums;
     const size_t floor_bytes = h->smem_per_sm / (blocks_per_sm + 1) - kSmemReserve + 1024;
     if (smem < floor_bytes && blocks_per_sm < max_blocks) smem = floor_bytes;

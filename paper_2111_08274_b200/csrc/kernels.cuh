@@ -1739,7 +1739,8 @@ k_round_rows(WT *__restrict__ w, MT *__restrict__ m, int64_t stride, int64_t n_p
 constexpr int kResidentThreads = 128;
 constexpr int kResidentMaxBlocks = 6;  // per SM: what the registers are bounded for (80 a thread; builds that use no more
                                        // than 72 could have 7); shared memory sets the actual number
-constexpr int kResidentOneVisitMaxBlocks = 5;  // ... of the build with one visit per row and round
+constexpr int kResidentOneVisitMaxBlocks = 5;  // ... of the build with one visit per row and round, as far as rows make
+                                               // room for each other: a sixth runs where there is room for as many rows
 
 struct ResidentBatch {
   int32_t n, k, n_rounds;
@@ -1849,8 +1850,9 @@ constexpr size_t resident_sums_bytes(int n, int rounds) {
 // hide latency with count for more, or with all rows on the SM, that costs more than it saves.  Sustained, us per
 // round of a batch of 8, apart / one visit: 16 devices, 2^24, one step 406 / 387, 2^22 112.4 / 107.3; 32 devices,
 // 2^22 300 / 282; 16 devices, 2^24, two steps 590 / 587; 14.7 M, steps 1,1,2,2,4,4,8,8 809 / 831; all rows on the SM, 8
-// devices, 11.2 M, one step 118 / 121; bf16 parameters, 16 devices, 2^22, one step 102 / 107.  With 6 blocks per SM
-// instead of 5: 2^24, one step 397.
+// devices, 11.2 M, one step 118 / 121; bf16 parameters, 16 devices, 2^22, one step 102 / 107.  Fewer rows on the SM for a
+// sixth block lose (2^24, one step 397), but where short batches' sums leave room for one with the same rows it gains; with 5
+// / 6: 16 devices, 2^24, 2 rounds, one step 511 / 490, 14 devices, 3 rounds 385 / 355, 9 devices, 4 rounds 236 / 218.
 enum class Resident { kAll, kPart, kPartOneVisit };
 constexpr int resident_max_blocks(Resident form) {
   return form == Resident::kPartOneVisit ? kResidentOneVisitMaxBlocks : kResidentMaxBlocks;
