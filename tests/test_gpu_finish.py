@@ -1,6 +1,7 @@
 """The last-block finish of the statistics and of the fused round at the sizes where its loops change
 shape: block counts around the group size (128 blocks), around a warp's stride over the partial sums
-(32 lanes x 4 loads), one block, and more than one group; a launch with one round and one with several.
+(32 lanes x 4 loads), one block, and more than one group; a launch with one round and one with several;
+finished by one block and in two levels.
 The sums must match a double-precision sum over the arena as it stands afterwards.  Bounds, all terms being
 positive: in the fused round a term is rounded at most 8 times in a thread's pack (each square is fused to the
 sum) and once across a pair of lanes, in the statistics kernel 16 times in a thread's chunk of 4 packs of 4;
@@ -50,7 +51,8 @@ def test_sums_over_block_counts(blocks, n, k, extra):
 
 @pytest.mark.parametrize("blocks,rounds", [(481, 1), (482, 1), (160, 3), (161, 3)])
 def test_one_group_and_several(blocks, rounds):
-    """17 devices: 34 sums per round and block on both sides of the 16,384 that one block adds alone."""
+    """17 devices, odd numbers of blocks and values: finished by one block (160 and 161 blocks, whatever the rounds; 481 and
+    482 with the 34 values of one round)."""
     wl = Workload("fin", 17, 2048 * blocks - 1, 5, 1, "fixed", (1,) * 17, grad_std=1e-2, seed=workloads.BASE_SEED + blocks)
     arena = runtime.Arena(wl)
     for first in (0, rounds):                            # the tickets are back at zero for the second launch
@@ -60,7 +62,7 @@ def test_one_group_and_several(blocks, rounds):
 
 
 @pytest.mark.parametrize("n,blocks,rounds", [(2, 512, 1), (2, 513, 1), (16, 512, 1), (17, 257, 1), (24, 256, 2), (24, 257, 2),
-                                             (24, 384, 2), (32, 512, 1), (32, 513, 1), (1, 1024, 1), (1, 1025, 1)])
+                                             (24, 383, 2), (24, 384, 2), (24, 385, 2), (32, 512, 1), (32, 513, 1), (1, 1024, 1), (1, 1025, 1)])
 def test_one_level_and_two(n, blocks, rounds):
     """Both sides of the lines between a finish by one block and one in two levels: 256 blocks, 512 blocks, and the number
     of values in between; in two levels with a last group of 128 blocks, of fewer and of one."""

@@ -20,10 +20,12 @@ def _gpu():
     require_gpu()
 
 
-# devices, parameters, rounds per call: row walk; a warp per row, alone and in a batch; rows on the SM, in a small
-# arena and with all and with a part of the rows of a large one
-FORMS = {"walk": (4, 140_001, 1), "rows": (4, 1_001, 1), "rows_batch": (4, 1_001, 3), "on_sm_small": (3, 1_500_007, 2),
-         "on_sm_all": (4, 9_400_003, 3), "on_sm_part": (16, 2_350_003, 2)}
+# devices, parameters, rounds per call: row walk; a warp per row, alone and in a batch, in blocks of up to 512 threads and
+# of more; rows on the SM, in a small arena and with all and with a part of the rows of a large one (with fp32 parameters
+# 16 devices take one visit per row, 9 visits apart)
+FORMS = {"walk": (4, 140_001, 1), "rows": (4, 1_001, 1), "rows_batch": (4, 1_001, 3), "rows_large": (32, 1_001, 1),
+         "rows_large_batch": (32, 1_001, 3), "on_sm_small": (3, 1_500_007, 2), "on_sm_all": (4, 9_400_003, 3),
+         "on_sm_part": (16, 2_350_003, 2), "on_sm_part_apart": (9, 4_200_003, 3)}
 
 
 def arena(n, P, storage, sync_every):
