@@ -2,7 +2,7 @@
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--workload c2]
                     [--min-seconds 0.5] [--sweep default|full|none] [--no-cpu-baseline]
-    python bench.py --table saved_line.json                               (markdown tables of its sweep)
+    python bench.py --table saved_line.json                        (markdown tables of a --sweep full line)
     python bench.py --profile-case [--pc-fused] [--pc-steps 1,8] ...      (target of ncu captures)
 
 A "step" is one round of the whole hot path over one synthetic workload: local update of every
@@ -28,7 +28,9 @@ per-replica statistics - one hadfl_round call, one kernel launch.  Prints ONE JS
   sweep     the metric against P: the bandwidth sweep (N=16, k=4, P = 2^20 .. 2^27, fp32 and bf16
             storage, one step per device and step ratios 1,1,2,2,4,4,8,8) plus the VGG-16- and
             ResNet-50-sized workloads: rounds/s of the fused round and GB/s of every kernel.
-            Outside the timed region; N = 1 only.
+            Outside the timed region; N = 1 only.  In the line by default as a short row per
+            workload, so that the line stays below 8,000 characters; --sweep full carries
+            everything that was measured.
   cpu_baseline  the CPU checker (single thread, as it stands) on a column sample of the same
             workload, scaled to the full vector; beside it the same sample on all host cores
             (the checker's -fopenmp build).
@@ -424,11 +426,24 @@ def run_sweep(peak, frac_key, which="default", rounds=12):
     return out, sync
 
 
+SHORT_COLUMNS = ["workload", "rounds_per_s", "one_round_per_launch", "separate_calls", "round_gbs"]
+
+
+def short_point(p):
+    """A point of the sweep as a short row, see SHORT_COLUMNS: rounds/s by calls of several rounds, with one round per
+    launch and as separate calls, and the algorithmic GB/s of the fused round."""
+    values = (p["rounds_per_s"], p["rounds_per_s_one_round_per_launch"], p["separate_calls_rounds_per_s"],
+              p["kernels"]["round"]["achieved_gbs"])
+    return [p["workload"]] + [float("%.4g" % v) for v in values]
+
+
 def print_tables(path):
     """Markdown tables of the sweep carried by a saved JSON line of this benchmark."""
     with open(path) as f:
         line = json.loads(f.read().strip().splitlines()[-1])
     sw = line["sweep"]
+    if "columns" in sw:
+        raise SystemExit("%s has the sweep's short rows only: save a line of --sweep full" % path)
     peak = sw["peak_gbs"]
     key = "frac_of_%s_hbm" % sw["peak_kind"]
 
@@ -588,6 +603,9 @@ def run_ours(args, wl):
     separate = {"rounds_per_s": world * 1e3 / sep_ms, "ms_per_round": sep_ms, "rounds": Ks,
                 "what": "hadfl_local_step + hadfl_select + hadfl_aggregate + hadfl_stats_enqueue"}
 
+    for entry in kernels.values():
+        del entry["traffic_is"]      # (in the roofline, once)
+
     # ---- roofline of the timed kernel -----------------------------------------------------------------
     sm_mhz = clocks["sm_mhz"] or SM_MAX_MHZ
     busiest = max(PIPE_CYCLES_PER_ELEM_STEP, key=PIPE_CYCLES_PER_ELEM_STEP.get)
@@ -696,6 +714,8 @@ def run_ours(args, wl):
         line["sweep"] = {"what": "fused round (rounds/s, one hadfl_round call per round, CUDA events) and "
                                  "every kernel's algorithmic GB/s against P; 12 rounds per point, medians",
                          "peak_gbs": peak, "peak_kind": peak_kind, "points": points}
+        if args.sweep != "full":
+            line["sweep"].update({"columns": SHORT_COLUMNS, "points": [short_point(p) for p in points]})
         if sync:
             line["sweep"]["sync"] = sync
     if rank == 0 and world == 1 and not args.no_cpu_baseline:

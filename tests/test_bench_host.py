@@ -66,3 +66,19 @@ def test_table_printer_reads_a_saved_line(bench, tmp_path, capsys):
     out = capsys.readouterr().out
     assert "| c5_p24_fp32 | 16 | 16777216 | 4 | fp32 | 1.00 |" in out and "5000 (77 / 62)" in out
     assert "| 1400 | 1500 (8) |" in out
+
+
+def test_the_default_sweep_is_short_rows(bench, tmp_path):
+    """A long line is not kept whole: 22 workloads in less than 1,500 characters."""
+    k = bench.gbs_entry(1e9, 0.2123456789, 6464.3, "frac_of_measured_hbm")
+    point = {"workload": "c5_p24_bf16_het", "rounds_per_s": 1512.3456789, "separate_calls_rounds_per_s": 1123.456789,
+             "rounds_per_s_one_round_per_launch": 1412.3456789, "kernels": {"round": k, "local_step": k}}
+    row = bench.short_point(point)
+    assert row == ["c5_p24_bf16_het", 1512.0, 1412.0, 1123.0, 4709.0] and len(row) == len(bench.SHORT_COLUMNS)
+    rows = [row] * len(bench.sweep_cases("default"))
+    assert len(json.dumps(rows)) < 1500
+    path = tmp_path / "line.json"
+    path.write_text(json.dumps({"sweep": {"peak_gbs": 6464.3, "peak_kind": "measured", "columns": bench.SHORT_COLUMNS,
+                                          "points": rows}}))
+    with pytest.raises(SystemExit):
+        bench.print_tables(str(path))
