@@ -362,7 +362,7 @@ int launch_local_step(hadfl_handle *h, const LocalStepArgs &a, float lr) {
 //   one round per launch: 8 devices 131,072: 12.7 / 12.0, 28.8 / 17.8; 200,000: 12.7 / 14.7, 29.1 / 22.9;
 //     16 devices 65,536: 18.0 / 12.4, 51.3 / 18.8; 131,072: 18.6 / 17.9, 51.6 / 28.8; 262,144: 18.8 / 26.8;
 //     32 devices 131,072 (16 selected): 31.1 / 37.2
-//   stochastic rounding (bf16 parameters and momentum; these builds spill 60 to 70 bytes a thread), one round: 8
+//   stochastic rounding (bf16 parameters and momentum; these builds spill about 100 bytes a thread), one round: 8
 //     devices 131,072: 22.5 / 14.0, 23.7 / 17.3 (uniform 1..8); 16 devices 131,072: 24.7 / 20.5, 41.8 / 28.2; 8 rounds:
 //     16 devices 262,144: 26.9 / 20.4, 45.1 / 34.8; 32 devices 131,072: 46.0 / 26.8, 86.6 / 44.3
 bool rows_form(const hadfl_handle *h, int n_rounds) {

@@ -21,7 +21,7 @@ pytestmark = pytest.mark.gpu
 HERE = os.path.dirname(os.path.abspath(__file__))
 SELECTION = ["test_gpu_round.py", "test_gpu_kernels.py", "test_gpu_rounding.py", "test_gpu_groups.py",
              "test_gpu_run.py", "test_zz_no_alloc.py", "test_gpu_round_rows.py", "test_gpu_rounds_resident.py",
-             "test_gpu_round_nonfinite.py", "test_gpu_unaligned_rows.py",
+             "test_gpu_round_nonfinite.py", "test_gpu_unaligned_rows.py", "test_gpu_finish.py", "test_gpu_stats_order.py",
              "test_gpu_configs.py::test_c1_full_arena_every_round",
              "test_gpu_configs.py::test_c1_ragged_tail_full_arena",
              "test_gpu_configs.py::test_c2_shrunk_full_arena",

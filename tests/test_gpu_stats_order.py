@@ -49,8 +49,9 @@ def test_row_walk(blocks):
 @pytest.mark.parametrize("tiles", [(64, 256), (1, 2), (2, 3), (3, 4), (5, 131), (63, 65), (128, 130), (37, 101)])
 @pytest.mark.parametrize("n,P", [(1, 37_889), (1, 131_072), (2, 30_001), (2, 100_001), (2, 131_071), (3, 37_888), (3, 113_663), (4, 30_000),
                                  (4, 37_889), (4, 100_000), (4, 131_072), (5, 113_664), (5, 113_665), (7, 70_001), (8, 37_889), (8, 75_776),
-                                 (8, 75_777), (16, 37_888)])
+                                 (8, 75_777), (8, 131_072), (16, 37_888), (16, 131_072), (24, 87_381), (32, 65_536)])
 def test_warp_per_row(n, P, tiles):
     """One to four tiles per block in a batch, where one round has eight, four, two or one: the most that an SM takes in
-    one block, one tile more, and in between."""
+    one block, one tile more, and in between.  Beyond that, the same blocks in both, up to 512, with a finish in one
+    level for one round and in two for several."""
     check_order(n, P, [min(256 * t + 8, P - 1) for t in tiles], (2, 5, 8))
