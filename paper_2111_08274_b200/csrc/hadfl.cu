@@ -400,7 +400,8 @@ int rows_groups(int n_devices) { return n_devices < 8 ? 8 / n_devices : 1; }
 // all 16 warps, for the finish.  Measured, us per round of a batch of 8, tiles for 8 warps / one block per SM / the same
 // without the warps for the finish: 4 devices, 100,000 parameters 3.54 / 2.83 / 2.95, 30,000 2.72 / 2.10 / 2.65; 2 devices,
 // 300,001 2.53 / 2.12 / 2.12, 30,000 1.78 / 1.42 / 2.07; 8 devices, 70,001 4.88 / 4.25; 16 devices, 37,000 5.38 / 5.17.
-// (1 and 2 devices: 4 tiles instead of 3, see rows_units.)
+// 1 and 2 devices take 4 tiles instead of 3, so that a single round's blocks hold whole ones of the batch's (rows_units):
+// 2 devices, 100,000 parameters 1.55 / 1.58 us per round of a batch of 8, 3.28 / 3.18 of 2, single rounds 5.5 / 4.8.
 int rows_groups_one_per_sm(const hadfl_handle *h) {
   const int n = h->cfg.n_devices;
   const int64_t most = kRowsFewThreads / 32 / n, tiles = rows_tiles(h->cfg.n_params);
